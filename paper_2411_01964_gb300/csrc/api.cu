@@ -90,8 +90,6 @@ sv_status cuda_status(cudaError_t e) { return e == cudaSuccess ? SV_OK : SV_ECUD
   DevGuard dev_guard__((c)->device);          \
   if (!dev_guard__.ok) return SV_ECUDA
 
-uint32_t ilog2_u32(uint32_t x) { return 31u - (uint32_t)__builtin_clz(x); }
-
 // Number of table primes p with p <= x.
 uint32_t primes_upto(const sv_ctx *c, uint64_t x) {
   if (x > 0xFFFFFFFFull) x = 0xFFFFFFFFull;
@@ -131,6 +129,13 @@ sv_status normalise_config(sv_ctx *c, sv_config *k) {
   return SV_OK;
 }
 
+// Margin words of the stream layout: the knob's margin, rounded up so that it
+// ends between two threads' runs.
+uint32_t stream_margin_words(const sv_config &k) {
+  const uint32_t mw = 1u << (k.margin_log2 - 6);
+  return (mw + kStreamMarginWords - 1) / kStreamMarginWords * kStreamMarginWords;
+}
+
 // Largest window span (bits) of any range of a launch.
 uint64_t max_span_bits(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
   uint64_t m = 0;
@@ -146,12 +151,22 @@ uint64_t max_span_bits(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
 // so it buckets every prime from kSegmentedLargeMin up (measured best on
 // single ranges of 2^34 and 2^36 integers: a sparse prime costs every tile
 // some work, a bucketed one only the tiles it strikes).
-Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges = 0) {
+// stream_threads: block size of the stream layout (streams.cu), 0 for the
+// linear one (tiles.cu).
+Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges = 0, uint32_t stream_threads = 0) {
   const sv_config &k = c->cfg;
   Geometry g{};
   g.tw = 1u << (k.tile_log2 - 5);
-  g.tw_log2 = ilog2_u32(g.tw);
   g.mw = 1u << (k.margin_log2 - 6);
+  g.threads = k.threads;
+  g.ctas = k.ctas_per_sm;
+  if (stream_threads) {
+    g.stream = 1;
+    g.threads = stream_threads;
+    g.mw = stream_margin_words(k);
+    g.tw = kStreamRun * stream_threads - g.mw;
+  }
+  g.tw_inv = ~0ull / g.tw;
   g.kwin = k.margin_log2;
   g.rec_t = k.record_k_threshold;
   g.i_med = k.stamp_primes;  // the stamped primes are the table's first entries
@@ -163,7 +178,7 @@ Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges 
   g.i_dense = i;
   // head: at least one strike per thread and window (struck with a stride of
   // one thread block); the rest of the dense primes share a numbering
-  const uint64_t head_q = 32ull * ((uint64_t)g.tw + g.mw) / (uint64_t)k.threads;
+  const uint64_t head_q = 32ull * ((uint64_t)g.tw + g.mw) / (uint64_t)g.threads;
   uint32_t h = g.i_med;
   while (h < g.i_dense && (uint64_t)c->h_p[h] * c->h_p[h] <= head_q) ++h;
   g.n_head = h - g.i_med;
@@ -192,8 +207,70 @@ Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges 
   g.bucket_auto = cap;
   if (k.bucket_capacity) cap = k.bucket_capacity;  // explicit override (grown on overflow)
   g.bucket_cap = cap;
+  if (g.stream) {  // resident blocks: as many threads as the configured shape has, as far as the shared memory goes
+    const size_t smem = stream_smem(g.threads, g.i_large - g.i_dense) + stream_static_smem() + 1024;
+    g.ctas = (uint32_t)std::min<size_t>((size_t)k.ctas_per_sm * k.threads / g.threads, (c->smem_optin + 1024) / smem);
+    g.ctas = std::max(g.ctas, 1u);
+  }
   g.stage_cap = k.list_stage_capacity ? std::min<uint32_t>(k.list_stage_capacity, kStageCap) : kStageCap;
   return g;
+}
+
+// The block size of the stream layout for a launch of `specs`, 0 if the
+// launch takes the linear tile kernel: that one has the per-n output, lists
+// of mink < 6, the unordered lists a launch falls back to, bitmaps in device
+// memory, other stamps than the four smallest primes, and block sizes other
+// than a thread per 2^10 odd n of the tile.
+// The tile knob gives the largest block.  A launch of few tiles takes smaller
+// ones, down to 64 threads, until there are two tiles per SM or no range
+// would be cut any more: a tile's time is nearly proportional to its
+// size, and SMs without a tile idle, but a smaller block only does the work of
+// an uncut short range with fewer threads.
+uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, const Workspace &ws) {
+  const sv_config &k = c->cfg;
+  if (k.record_k_threshold <= 5 || ws.force_general || k.stamp_primes != 4 || k.tile_log2 < 15 || k.tile_log2 > 19 ||
+      k.threads != 1u << (k.tile_log2 - 10) || !c->d_stamp)
+    return 0;
+  uint64_t bits = 0, longest = 0;
+  for (const RangeSpec &s : specs) {
+    if (s.d_per_n || s.sieve_only || s.bitmap_in) return 0;
+    if (s.hi <= s.lo) continue;
+    bits += (s.hi - s.lo) / 2;
+    longest = std::max(longest, (s.hi - s.lo) / 2);
+  }
+  const uint64_t margin = 32ull * stream_margin_words(k);
+  uint32_t S = k.threads;
+  if (margin * 8 > 32ull * kStreamRun * S) return 0;  // the margin would be most of the window
+  if (stream_smem(S, kMaxSparsePrimes) + stream_static_smem() + 1024 > c->smem_optin) return 0;
+  while (S > 64 && margin * 16 <= 32ull * kStreamRun * S / 2 && longest + margin > 32ull * kStreamRun * S / 2 &&
+         specs.size() + bits / (32ull * kStreamRun * S - margin) < 2ull * (uint64_t)c->num_sms)
+    S /= 2;
+  return S;
+}
+
+// The geometry of one launch, with the bucket depth earlier launches grew to.
+Geometry geometry_of(const sv_ctx *c, const std::vector<RangeSpec> &specs, const Workspace &ws) {
+  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size(), stream_threads(c, specs, ws));
+  if (ws.bucket_cap > g.bucket_cap) g.bucket_cap = ws.bucket_cap;
+  return g;
+}
+
+// Launches the tile kernel of the launch's geometry; max_tiles bounds the
+// grid.
+cudaError_t launch_tile_stage(const sv_ctx *c, const TileArgs &t, int mode, bool search_all, uint32_t max_tiles,
+                              cudaStream_t st) {
+  const Geometry &g = t.g;
+  const uint32_t grid = std::min((uint32_t)c->num_sms * g.ctas, max_tiles);
+  if (!g.stream) return launch_tiles(t, g.threads, grid, 4ull * (g.tw + g.mw), mode, st);
+  StreamArgs s;
+  std::memset(&s, 0, sizeof(s));
+  s.t = t;
+  s.stamp = c->d_stamp;
+  s.magic = stream_magic(kStreamRun * g.threads);
+  s.sparse_room = g.i_large - g.i_dense;
+  s.search_all = search_all ? 1u : 0u;
+  plan_strikes(c->h_p.data() + g.i_med, g.i_dense - g.i_med, s.sparse_room, g.threads, &s.plan);
+  return launch_stream_tiles(s, grid, st);
 }
 
 // p_hyb^2: multiples j p^2 with p >= p_hyb are enumerated by j (0: none)
@@ -216,6 +293,7 @@ sv_status ensure_tile_smem(sv_ctx *c) {
   const size_t smem = 4ull * ((1ull << (c->cfg.tile_log2 - 5)) + (1ull << (c->cfg.margin_log2 - 6)));
   if (smem > c->smem_set.load()) {
     SV_TRY_CUDA(tile_kernel_setup(smem));
+    SV_TRY_CUDA(stream_kernel_setup((int)c->smem_optin));
     c->smem_set.store(smem);
   }
   return SV_OK;
@@ -418,12 +496,9 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
       t.stage_k = ws.stage_k.p;
       t.stage_cnt = ws.stage_cnt.p;
     }
-    const size_t smem = 4ull * (g.tw + g.mw);
-    uint32_t grid = (uint32_t)c->num_sms * c->cfg.ctas_per_sm;
-    if (grid > ws.total_tiles) grid = ws.total_tiles;
     {
       KTimer kt(c, ws.tile_kernel_id, st);
-      SV_TRY_CUDA(launch_tiles(t, c->cfg.threads, grid, smem, mode, st));
+      SV_TRY_CUDA(launch_tile_stage(c, t, mode, ws.search_all, ws.total_tiles, st));
       kt.done();
     }
     c->launches++;
@@ -443,7 +518,8 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
       s.stage_k = ws.stage_k.p;
       s.stage_cnt = ws.stage_cnt.p;
       s.stage_cap = g.stage_cap;
-      s.tw_log2 = g.tw_log2;
+      s.tw = g.tw;
+      s.tw_inv = g.tw_inv;
     }
     {
       KTimer kt(c, kKStrag, st);
@@ -495,10 +571,9 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
                         ws.stage_cnt.p};
   std::memcpy(key.p, ptrs, sizeof(ptrs));
   key.g = g;
-  key.threads = c->cfg.threads;
-  key.ctas = c->cfg.ctas_per_sm;
   key.mode = (uint32_t)mode;
   key.strag_cap = ws.strag_cap;
+  key.search_all = ws.search_all ? 1u : 0u;
   key.req_copy = req_copy;
   key.n_table = c->n_primes;
   // per-kernel timing of the tile kernel: event-record nodes around it
@@ -551,7 +626,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
         t.stage_cnt = ws.stage_cnt.p;
       }
       if (timed) e = cudaEventRecordWithFlags(ws.gev[0], st, cudaEventRecordExternal);
-      if (!e) e = launch_tiles(t, c->cfg.threads, (uint32_t)c->num_sms * c->cfg.ctas_per_sm, 4ull * (g.tw + g.mw), mode, st);
+      if (!e) e = launch_tile_stage(c, t, mode, ws.search_all, 0xFFFFFFFFu, st);
       if (!e && timed) e = cudaEventRecordWithFlags(ws.gev[1], st, cudaEventRecordExternal);
     }
     if (!e) {
@@ -571,7 +646,8 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
         sa.stage_k = ws.stage_k.p;
         sa.stage_cnt = ws.stage_cnt.p;
         sa.stage_cap = g.stage_cap;
-        sa.tw_log2 = g.tw_log2;
+        sa.tw = g.tw;
+        sa.tw_inv = g.tw_inv;
       }
       e = launch_stragglers(sa, (uint32_t)c->num_sms * 2, st);
     }
@@ -666,7 +742,7 @@ void sort_by_n(const uint64_t *ns, const uint8_t *ks, uint64_t cnt, uint64_t lo,
       for (uint32_t x = i; x > start[b] && out[x - 1].first > out[x].first; --x) std::swap(out[x - 1], out[x]);
 }
 
-enum Collect { kDone, kRetryBucket, kRetryStrag, kRetryList, kRetryGeneral };
+enum Collect { kDone, kRetryBucket, kRetryStrag, kRetryList, kRetryGeneral, kRetryFirst };
 constexpr uint64_t kSpeculativeList = 1ull << 18;  // list entries copied without waiting for the count
 
 // How many list entries the consumer of range r can take: its result buffer,
@@ -739,6 +815,15 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
     *what = kRetryGeneral;
     return SV_OK;
   }
+  // a k <= 5 that occurs, but not in its range's first tile: the stream layout
+  // searched only that one for its first n
+  if (ws.ordered && !ws.search_all)
+    for (uint32_t r = 0; r < n; ++r)
+      for (int k = 1; k <= 5; ++k)
+        if (ws.h_slots.p[r].hist[k] && ws.h_slots.p[r].first_n[k] == kNoN) {
+          *what = kRetryFirst;
+          return SV_OK;
+        }
   // an unordered list that the device truncated is re-run with exact room,
   // so that the caller receives the smallest entries, deterministically; an
   // ordered list already holds the smallest ones and is re-run only when
@@ -866,9 +951,8 @@ sv_status run_ranges(sv_ctx *c, std::vector<RangeSpec> &specs, sv_range_result *
                      Workspace &ws, bool graph) {
   sv_status s = ensure_tile_smem(c);
   if (s) return s;
-  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size());
-  if (ws.bucket_cap > g.bucket_cap) g.bucket_cap = ws.bucket_cap;
   for (int attempt = 0; attempt < 8; ++attempt) {
+    const Geometry g = geometry_of(c, specs, ws);
     if ((s = plan(c, specs, g, ws))) return s;
     if ((s = graph ? enqueue_graph(c, g, ws, st) : enqueue(c, g, ws, st))) return s;
     Collect what;
@@ -876,14 +960,12 @@ sv_status run_ranges(sv_ctx *c, std::vector<RangeSpec> &specs, sv_range_result *
     if (what == kDone) {
       c->last_h2d = ws.h2d_bytes;
       c->last_d2h = ws.d2h_bytes;
-      ws.force_general = false;
+      ws.force_general = ws.search_all = false;
       return SV_OK;
     }
     if (what == kRetryGeneral) ws.force_general = true;
-    if (what == kRetryBucket) {
-      g.bucket_cap = std::max<uint32_t>(g.bucket_cap * 4, g.bucket_auto);
-      ws.bucket_cap = g.bucket_cap;
-    }
+    if (what == kRetryFirst) ws.search_all = true;
+    if (what == kRetryBucket) ws.bucket_cap = std::max<uint32_t>(g.bucket_cap * 4, g.bucket_auto);
     if (what == kRetryStrag) ws.strag_cap *= 4;
     if (what == kRetryList) {
       for (uint32_t r = 0; r < specs.size(); ++r) {
@@ -1002,7 +1084,7 @@ sv_status run_plain(sv_ctx *c, std::vector<RangeSpec> &sieve, std::vector<RangeS
     if (what == kDone) {
       c->last_h2d = c->ws.h2d_bytes + (sieve.empty() ? 0 : c->ws_sieve.h2d_bytes);
       c->last_d2h = c->ws.d2h_bytes + (sieve.empty() ? 0 : c->ws_sieve.d2h_bytes);
-      c->ws.force_general = false;
+      c->ws.force_general = c->ws.search_all = false;
       return SV_OK;
     }
     plain_retry(c, what, sr, sieve, scan, out);
@@ -1013,8 +1095,7 @@ sv_status run_plain(sv_ctx *c, std::vector<RangeSpec> &sieve, std::vector<RangeS
 sv_status launch_ranges_async(sv_ctx *c, std::vector<RangeSpec> &specs, Workspace &ws, cudaStream_t st) {
   sv_status s = ensure_tile_smem(c);
   if (s) return s;
-  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size());
-  if (ws.bucket_cap > g.bucket_cap) g.bucket_cap = ws.bucket_cap;
+  const Geometry g = geometry_of(c, specs, ws);
   if ((s = plan(c, specs, g, ws))) return s;
   return enqueue_graph(c, g, ws, st);
 }
@@ -1024,10 +1105,11 @@ sv_status collect_ranges(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_rang
   Collect what;
   sv_status s = collect(c, specs, outs, ws, st, &what);
   *retry = (what != kDone);
-  if (what == kDone) ws.force_general = false;
+  if (what == kDone) ws.force_general = ws.search_all = false;
   if (what == kRetryGeneral) ws.force_general = true;
+  if (what == kRetryFirst) ws.search_all = true;
   if (what == kRetryBucket)
-    ws.bucket_cap = std::max<uint32_t>(ws.bucket_cap * 4, make_geometry(c, max_span_bits(c, specs), specs.size()).bucket_auto);
+    ws.bucket_cap = std::max<uint32_t>(ws.bucket_cap * 4, geometry_of(c, specs, ws).bucket_auto);
   if (what == kRetryStrag) ws.strag_cap *= 4;
   return s;
 }
@@ -1147,6 +1229,7 @@ void sv_destroy(sv_ctx *c) {
   cudaFree(c->d_inv);
   cudaFree(c->d_lim);
   cudaFree(c->d_pbits);
+  cudaFree(c->d_stamp);
   for (auto &k : c->kev) {
     cudaEventDestroy(k.a);
     cudaEventDestroy(k.b);
@@ -1176,13 +1259,29 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
   cudaError_t e = build_prime_table(pmax, &d_p, &d_mu, &d_inv, &d_lim, &d_bits, &bits_words, &n, &n_div, c->stream);
   if (e == cudaErrorMemoryAllocation) return SV_ENOMEM;
   if (e != cudaSuccess) return SV_ECUDA;
-  std::vector<uint32_t> hp(n);
-  if (n && cudaMemcpy(hp.data(), d_p, 4ull * n, cudaMemcpyDeviceToHost) != cudaSuccess) {
+  auto free_table = [&] {
     cudaFree(d_p);
     cudaFree(d_mu);
     cudaFree(d_inv);
     cudaFree(d_lim);
     cudaFree(d_bits);
+  };
+  if (!c->d_stamp) {  // the stream layout's stamp tables (they depend on nothing)
+    uint32_t *d_stamp = nullptr;
+    if (cudaMalloc((void **)&d_stamp, 4ull * kStreamStampStride * kStreamSizes) != cudaSuccess) {
+      free_table();
+      return SV_ENOMEM;
+    }
+    c->d_stamp = d_stamp;
+    if (launch_stamp_tables(d_stamp, c->stream) != cudaSuccess) {
+      free_table();
+      return SV_ECUDA;
+    }
+    c->launches += kStreamSizes;
+  }
+  std::vector<uint32_t> hp(n);
+  if (n && cudaMemcpy(hp.data(), d_p, 4ull * n, cudaMemcpyDeviceToHost) != cudaSuccess) {
+    free_table();
     return SV_ECUDA;
   }
   cudaStreamSynchronize(c->stream);
@@ -1313,8 +1412,7 @@ sv_status sv_launch_batch(sv_ctx *c, const uint64_t *lo, const uint64_t *hi, siz
                                           c->cfg.list_capacity);
     specs[i].fail_cap = 16;
   }
-  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size());
-  if (c->ws.bucket_cap > g.bucket_cap) g.bucket_cap = c->ws.bucket_cap;
+  const Geometry g = geometry_of(c, specs, c->ws);
   if ((s = plan(c, specs, g, c->ws))) return s;
   if ((s = enqueue_graph(c, g, c->ws, c->stream))) return s;
   c->pending = true;
@@ -1337,9 +1435,10 @@ sv_status sv_fetch_batch(sv_ctx *c, sv_range_result *out, size_t count) {
   if (s) return s;
   if (what != kDone) {
     std::vector<RangeSpec> specs = c->pending_specs;
-    if (what == kRetryBucket) c->ws.bucket_cap = make_geometry(c, max_span_bits(c, specs), specs.size()).bucket_cap * 4;
+    if (what == kRetryBucket) c->ws.bucket_cap = geometry_of(c, specs, c->ws).bucket_cap * 4;
     if (what == kRetryStrag) c->ws.strag_cap *= 4;
     if (what == kRetryGeneral) c->ws.force_general = true;
+    if (what == kRetryFirst) c->ws.search_all = true;
     s = run_ranges(c, specs, outs.data(), c->stream, c->ws, true);
   }
   return s;
@@ -1399,8 +1498,7 @@ sv_status sv_launch_range(sv_ctx *c, uint64_t lo, uint64_t hi, uint8_t *d_per_n_
   specs[0].d_per_n = d_per_n_k;
   specs[0].list_cap = c->cfg.list_capacity;
   specs[0].fail_cap = 1024;
-  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size());
-  if (c->ws.bucket_cap > g.bucket_cap) g.bucket_cap = c->ws.bucket_cap;
+  const Geometry g = geometry_of(c, specs, c->ws);
   if ((s = plan(c, specs, g, c->ws))) return s;
   // the captured graph (fewer launch gaps), unless a kernel other than the
   // tile kernel is being timed: a graph brackets only the tile kernel
@@ -1428,7 +1526,7 @@ sv_status sv_fetch_range(sv_ctx *c, sv_range_result *out) {
       plain_retry(c, what, sr, c->pending_sieve_specs, c->pending_specs, out);
       return run_plain(c, c->pending_sieve_specs, c->pending_specs, out, c->stream);
     }
-    c->ws.force_general = false;
+    c->ws.force_general = c->ws.search_all = false;
     c->last_h2d = c->ws.h2d_bytes + c->ws_sieve.h2d_bytes;
     c->last_d2h = c->ws.d2h_bytes + c->ws_sieve.d2h_bytes;
     return SV_OK;
@@ -1440,9 +1538,10 @@ sv_status sv_fetch_range(sv_ctx *c, sv_range_result *out) {
   if (what != kDone) {
     // an overflow: repeat the range with grown buffers, blocking
     std::vector<RangeSpec> specs = c->pending_specs;
-    if (what == kRetryBucket) c->ws.bucket_cap = make_geometry(c, max_span_bits(c, specs), specs.size()).bucket_cap * 4;
+    if (what == kRetryBucket) c->ws.bucket_cap = geometry_of(c, specs, c->ws).bucket_cap * 4;
     if (what == kRetryStrag) c->ws.strag_cap *= 4;
     if (what == kRetryGeneral) c->ws.force_general = true;
+    if (what == kRetryFirst) c->ws.search_all = true;
     s = run_ranges(c, specs, outs, c->stream, c->ws, false);
     if (s) return s;
   }
@@ -1593,8 +1692,7 @@ sv_status time_launch(sv_ctx *c, const std::vector<RangeSpec> &specs0, double *b
   }
   double best = 1e300;
   for (int rep = 0; rep < 3 && !s; ++rep) {
-    Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size());
-    if (c->ws.bucket_cap > g.bucket_cap) g.bucket_cap = c->ws.bucket_cap;
+    const Geometry g = geometry_of(c, specs, c->ws);
     if ((s = plan(c, specs, g, c->ws))) break;
     if (cudaEventRecord(a, c->stream) != cudaSuccess) s = SV_ECUDA;
     if (!s) s = enqueue_graph(c, g, c->ws, c->stream);
@@ -1693,7 +1791,7 @@ sv_status tune(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_config *chosen
     }
     {  // bucket depth: the automatic estimate, or twice it
       c->cfg = best;
-      const uint32_t cap_auto = make_geometry(c, max_span_bits(c, specs), specs.size()).bucket_auto;
+      const uint32_t cap_auto = geometry_of(c, specs, c->ws).bucket_auto;
       for (uint32_t v : {0u, 2u * cap_auto}) {
         if (s) break;
         sv_config k = best;

@@ -57,7 +57,7 @@ __device__ __forceinline__ BucketHit bucket_hit(const BucketArgs &a, uint64_t J,
   BucketHit h;
   const int64_t w = (int64_t)(J >> 5);
   uint32_t t = 0;
-  if (w >= w0) t = (uint32_t)((uint64_t)(w - w0) >> a.g.tw_log2);
+  if (w >= w0) t = (uint32_t)tile_index((uint64_t)(w - w0), a.g.tw, a.g.tw_inv);
   if (t >= n_tiles) t = n_tiles - 1;  // cannot happen: J < E
   const int64_t wst = w0 + (int64_t)t * a.g.tw - (int64_t)a.g.mw;
   h.t0 = tile_base + t;

@@ -75,7 +75,7 @@ struct RangeSpec {
 struct GraphKey {
   const void *p[16];
   Geometry g;
-  uint32_t threads, ctas, mode, strag_cap;
+  uint32_t mode, strag_cap, search_all;
   uint64_t req_copy;
   uint32_t n_table;
   uint32_t timed;  // 1: event-record nodes bracket the tile kernel
@@ -114,6 +114,7 @@ struct Workspace {
   bool any_per_n = false;
   bool ordered = false;        // the planned launch produces ordered lists (tile kernel mode 0)
   bool force_general = false;  // repeat with the unordered list path (a tile's staging overflowed)
+  bool search_all = false;     // repeat with the first occurrences of k <= 5 searched in every tile
   bool all_from_bitmap = false;  // every range reads its windows from a bitmap: no bucket fill
   int tile_kernel_id = 2;        // per-kernel timing id of this workspace's tile kernel launches
   uint64_t j_max = 0;  // largest odd-multiplier count of the launch (bucket fill by j)
@@ -172,6 +173,7 @@ struct sv_ctx {
   uint64_t *d_mu = nullptr, *d_inv = nullptr, *d_lim = nullptr;
   uint32_t *d_pbits = nullptr;  // odd-prime bitmap of the table's range
   uint64_t pbits_words = 0;
+  uint32_t *d_stamp = nullptr;  // the stream layout's stamp tables (streams.cu)
   uint32_t n_primes = 0, n_div = 0;
   std::vector<uint32_t> h_p;
   std::vector<uint32_t> h_pi;  // h_pi[b] = number of h_p entries below b * 2^kPiBlockLog2

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) straggler_kernel(StragArgs a) {
         if (k >= a.rec_t) {
           if (a.stage_n) {
             // ordered lists: join the staged entries of the tile holding n
-            const uint64_t t = ((((st.n - 1) >> 1) >> 5) - (uint64_t)R.w0) >> a.tw_log2;
+            const uint64_t t = tile_index((((st.n - 1) >> 1) >> 5) - (uint64_t)R.w0, a.tw, a.tw_inv);
             if (t < R.n_tiles) {
               const uint32_t gt = R.tile_base + (uint32_t)t;
               const uint32_t e = atomicAdd(&a.stage_cnt[gt], 1u);

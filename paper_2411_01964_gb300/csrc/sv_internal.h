@@ -126,8 +126,8 @@ struct LaunchHeader {
 };
 
 struct Geometry {
-  uint32_t tw;        // core words per tile (2^(tile_log2 - 5))
-  uint32_t mw;        // look-back words (2^(margin_log2 - 6))
+  uint32_t tw;        // core words per tile (2^(tile_log2 - 5); the stream layout: the window less the margin)
+  uint32_t mw;        // look-back words (2^(margin_log2 - 6); the stream layout: at least that)
   uint32_t kwin;      // largest k decided inside a window (= margin_log2)
   uint32_t rec_t;     // record threshold T
   uint32_t i_med;     // first prime index struck per tile (after the stamped ones)
@@ -135,13 +135,28 @@ struct Geometry {
   uint32_t n_head;    // the first n_head of them hit a window at least once per thread
   uint32_t i_large;   // primes >= i_large come through buckets
   uint32_t bucket_cap;
-  uint32_t tw_log2;   // log2(tw)
+  uint32_t stream;    // 1: the tile kernel of streams.cu
   uint32_t bucket_auto;  // host only: the automatic capacity estimate
   uint32_t i_hyb;     // primes >= i_hyb reach the buckets by enumerating odd multipliers j
   uint32_t p_hyb;     // the prime at i_hyb (0xFFFFFFFF: none)
   uint32_t stage_cap; // usable staged list entries per tile (<= kStageCap)
+  uint32_t threads;   // threads per block of the tile kernel
+  uint32_t ctas;      // its resident blocks per SM
   uint32_t pad;
+  uint64_t tw_inv;    // floor((2^64 - 1) / tw), for tile_index
 };
+
+// The tile holding the dw-th word of a range: dw / tw (the estimate is at
+// most one low for dw < 2^63).
+__host__ __device__ inline uint64_t tile_index(uint64_t dw, uint32_t tw, uint64_t tw_inv) {
+#ifdef __CUDA_ARCH__
+  uint64_t t = __umul64hi(dw, tw_inv);
+#else
+  uint64_t t = (uint64_t)(((unsigned __int128)dw * tw_inv) >> 64);
+#endif
+  if (dw - t * tw >= tw) ++t;
+  return t;
+}
 
 struct TileArgs {
   PrimeTab pt;
@@ -187,7 +202,8 @@ struct StragArgs {
   uint8_t *stage_k;
   uint32_t *stage_cnt;
   uint32_t stage_cap;
-  uint32_t tw_log2;
+  uint32_t tw;          // words per tile
+  uint64_t tw_inv;
 };
 
 // The ordered list (mode 0): each range's staged entries, tile by tile and
@@ -221,6 +237,40 @@ cudaError_t launch_tiles(const TileArgs &a, uint32_t threads, uint32_t grid, siz
                          cudaStream_t st);
 cudaError_t tile_kernel_setup(size_t smem);
 size_t tile_static_smem();
+
+// ---- the stream layout (streams.cu) -------------------------------------------
+constexpr uint32_t kStreamRun = 36;         // words per thread; the window has kStreamRun * threads words
+constexpr uint32_t kStreamMinThreads = 32;  // block sizes 32 * 2^j, j < kStreamSizes
+constexpr uint32_t kStreamSizes = 5;
+constexpr uint32_t kStreamStampStride = 2704;  // words per stamp table (one table per block size)
+constexpr uint32_t kStreamMarginWords = 9;  // the margin is a multiple of 9 words = 288 bits, so that it ends
+                                            // between two threads' runs
+// A warp's piece of one dense prime's strikes: steps m0 .. m0 + n - 1 of 32
+// strikes each.
+constexpr uint32_t kMaxStrikeTasks = 160, kMaxStrikeWarps = 16;
+struct StrikeTask {
+  uint16_t m0;
+  uint8_t d, n;
+};
+struct StrikePlan {
+  StrikeTask task[kMaxStrikeTasks];
+  uint8_t start[kMaxStrikeWarps + 1];  // warp w has tasks [start[w], start[w + 1])
+};
+struct StreamArgs {
+  TileArgs t;
+  const uint32_t *stamp;   // kStreamSizes stamp tables
+  uint32_t magic;          // stream_magic of the window's words
+  uint32_t sparse_room;    // sparse primes the block has room for (>= i_large - i_dense)
+  uint32_t search_all;     // 1: every tile searches the first occurrences of k <= 5, not only a range's first
+  StrikePlan plan;
+};
+cudaError_t launch_stamp_tables(uint32_t *d_tables, cudaStream_t st);
+void plan_strikes(const uint32_t *primes, uint32_t nd, uint32_t n_sparse, uint32_t threads, StrikePlan *plan);
+uint32_t stream_magic(uint32_t M);
+size_t stream_smem(uint32_t threads, uint32_t sparse_room);
+size_t stream_static_smem();
+cudaError_t stream_kernel_setup(int optin);
+cudaError_t launch_stream_tiles(const StreamArgs &s, uint32_t grid, cudaStream_t st);
 cudaError_t launch_stragglers(const StragArgs &a, uint32_t grid, cudaStream_t st);
 cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out,
                           uint32_t grid, cudaStream_t st);
