@@ -1118,10 +1118,7 @@ sv_status launch_points_async(sv_ctx *c, uint64_t count, Workspace &ws, cudaStre
   if (count == 0) return SV_OK;
   if (ws.points.ensure(count) || ws.points_out.ensure(count)) return SV_ENOMEM;
   SV_TRY_CUDA(cudaMemcpyAsync(ws.points.p, ws.h_points.p, 8 * count, cudaMemcpyHostToDevice, st));
-  uint64_t grid = (count * 32 + 255) / 256;
-  const uint64_t gmax = (uint64_t)c->num_sms * 8;
-  if (grid > gmax) grid = gmax;
-  SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)grid, st));
+  SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)c->num_sms, st));
   c->launches++;
   SV_TRY_CUDA(cudaMemcpyAsync(ws.h_points_out.p, ws.points_out.p, count, cudaMemcpyDeviceToHost, st));
   return SV_OK;
@@ -1137,13 +1134,9 @@ sv_status run_points(sv_ctx *c, const uint64_t *points, size_t count, uint8_t *o
     return SV_ENOMEM;
   std::memcpy(ws.h_points.p, points, 8 * count);
   SV_TRY_CUDA(cudaMemcpyAsync(ws.points.p, ws.h_points.p, 8 * count, cudaMemcpyHostToDevice, st));
-  uint64_t warps = count;
-  uint64_t grid = (warps * 32 + 255) / 256;
-  const uint64_t gmax = (uint64_t)c->num_sms * 8;
-  if (grid > gmax) grid = gmax;
   {
     KTimer kt(c, kKPoints, st);
-    SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)grid, st));
+    SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)c->num_sms, st));
     kt.done();
   }
   c->launches++;
@@ -1460,10 +1453,7 @@ sv_status sv_min_k_device(sv_ctx *c, const uint64_t *d_points, size_t count, uin
   if (count == 0) return SV_OK;
   SV_ON_DEVICE(c);
   std::lock_guard<std::mutex> lk(c->mu);
-  uint64_t grid = ((uint64_t)count * 32 + 255) / 256;
-  const uint64_t gmax = (uint64_t)c->num_sms * 8;
-  if (grid > gmax) grid = gmax;
-  if (launch_points(prime_tab(c), d_points, count, d_out_k, (uint32_t)grid, c->stream) != cudaSuccess)
+  if (launch_points(prime_tab(c), d_points, count, d_out_k, (uint32_t)c->num_sms, c->stream) != cudaSuccess)
     return SV_ECUDA;
   c->launches++;
   return SV_OK;

@@ -13,6 +13,8 @@
 // prime table; the warp stops at the first p with p^2 | s.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "strike.h"
 #include "sv_internal.h"
 
@@ -115,23 +117,241 @@ cudaError_t launch_stragglers(const StragArgs &a, uint32_t grid, cudaStream_t st
   return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) points_kernel(PrimeTab pt, const uint64_t *pts, uint64_t count,
-                                                     uint8_t *out) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t gw = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t e = gw; e < count; e += nw) {
+// ---- point queries -------------------------------------------------------------
+// Both kernels test a prime with the high word of t = s p^-1 mod 2^64 alone:
+// p | s means t <= lim, hence t_hi <= lim_hi; the rare candidates (and the
+// rarer false ones, t_hi = lim_hi) are decided with both words.  That is
+// three multiplies and a compare per prime and value.  Primes somewhat past
+// the cube root of s may be tested too: dividing one out leaves r = 1, a
+// prime, or (r = p^2) finds p^2 | s, so the test stays exact.
+__device__ __forceinline__ bool maybe_divides(uint64_t s, uint64_t inv, uint32_t lim_hi) {
+  const uint32_t s0 = (uint32_t)s, s1 = (uint32_t)(s >> 32), i0 = (uint32_t)inv, i1 = (uint32_t)(inv >> 32);
+  return __umulhi(s0, i0) + s0 * i1 + s1 * i0 <= lim_hi;
+}
+
+__device__ __forceinline__ uint32_t lim_high(const PrimeTab &pt, uint32_t i) {
+  return reinterpret_cast<const uint32_t *>(pt.lim)[2u * i + 1u];  // little endian
+}
+
+// r = s less its prime divisors up to the cube root: squarefree unless r is a
+// square above 1
+__device__ __forceinline__ bool cofactor_squarefree(uint64_t r) {
+  if (r == 1) return true;
+  const uint64_t x = isqrt_u64(r);
+  return x * x != r;
+}
+
+constexpr uint32_t kMaxDivisors = 16;  // a product of 16 odd primes exceeds 2^62
+
+// Few points: a block per point, its threads striding the primes, and K
+// exponents at a time, so that one pass over the primes mostly suffices.
+template <int K>
+__global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const uint64_t *pts, uint64_t count,
+                                                            uint8_t *out) {
+  __shared__ uint32_t bad, n_div[K];   // bad: bit j, p^2 divides the j-th value
+  __shared__ uint64_t div_inv[K][kMaxDivisors];
+  __shared__ uint32_t found;
+  const uint32_t tid = threadIdx.x, T = blockDim.x;
+  for (uint64_t e = blockIdx.x; e < count; e += gridDim.x) {
     const uint64_t n = pts[e];
     uint32_t k = 0;
-    if (n >= 3 && (n & 1ull)) k = warp_min_k_from(n, 1, pt);
-    if (lane == 0) out[e] = (uint8_t)k;
+    if (n >= 3 && (n & 1ull)) {
+      for (uint32_t k0 = 1;; k0 += K) {
+        __syncthreads();  // the previous round's results have been read
+        if (tid == 0) {
+          bad = 0;
+          found = k0 < 63 && (1ull << k0) < n ? 0u : (uint32_t)kFailK;
+        }
+        if (tid < K) n_div[tid] = 0;
+        __syncthreads();
+        if (found) break;  // no exponent left
+        uint64_t s[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          const uint32_t kj = k0 + (uint32_t)j;
+          s[j] = kj < 63 && (1ull << kj) < n ? n - (1ull << kj) : 1ull;  // (1: never the answer, see below)
+        }
+        for (uint32_t base = 0; base < pt.n_div; base += T) {
+          const uint64_t pb = pt.p[base];
+          if (pb * pb * pb > n) break;  // primes ascend (p < 2^21: no overflow)
+          const uint32_t i = base + tid;
+          if (i >= pt.n_div) continue;
+          const uint64_t inv = pt.inv[i];
+          const uint32_t lh = lim_high(pt, i);
+          bool any = false;
+#pragma unroll
+          for (int j = 0; j < K; ++j) any |= maybe_divides(s[j], inv, lh);
+          if (any) {
+            const uint64_t lim = pt.lim[i];
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+              const uint64_t t = s[j] * inv;
+              if (t > lim) continue;
+              if (t * inv <= lim) atomicOr(&bad, 1u << j);
+              const uint32_t d = atomicAdd(&n_div[j], 1u);
+              if (d < kMaxDivisors) div_inv[j][d] = inv;
+            }
+          }
+        }
+        __syncthreads();
+        if (tid < 32) {  // lane j decides the j-th value
+          bool ok = false;
+          const uint32_t j = tid, kj = k0 + j;
+          if (j < (uint32_t)K && kj < 63 && (1ull << kj) < n && !((bad >> j) & 1u)) {
+            uint64_t r = n - (1ull << kj);
+            for (uint32_t d = 0; d < min(n_div[j], kMaxDivisors); ++d) r *= div_inv[j][d];  // exact divisions
+            ok = cofactor_squarefree(r);
+          }
+          const uint32_t bal = __ballot_sync(0xFFFFFFFFu, ok);
+          if (tid == 0 && bal) found = k0 + (uint32_t)__ffs(bal) - 1u;
+        }
+        __syncthreads();
+        if (found) break;
+      }
+      k = found;
+    }
+    if (tid == 0) out[e] = (uint8_t)k;
+    __syncthreads();  // found is read above before the next point resets it
   }
 }
 
-cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t grid,
+// Many points: a warp takes kSlots points at a time and walks the primes once
+// for all of them (one load per prime for kSlots tests).  The first 32 primes,
+// which decide nearly every value that is not squarefree, come first and
+// alone: each slot's exponent advances until its value passes them.
+constexpr int kSlots = 4;
+__global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uint64_t *pts, uint64_t count,
+                                                          uint8_t *out) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t gw = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+  const uint64_t small_p = lane < pt.n_div ? pt.p[lane] : 0ull;
+  const uint64_t small_inv = lane < pt.n_div ? pt.inv[lane] : 0ull, small_lim = lane < pt.n_div ? pt.lim[lane] : 0ull;
+  uint64_t s[kSlots], r[kSlots], e[kSlots];  // value, its cofactor so far, point index
+  uint32_t k[kSlots];                        // exponent under test; 0: the slot takes a new point
+  uint64_t next = gw;
+#pragma unroll
+  for (int j = 0; j < kSlots; ++j) k[j] = 0, s[j] = r[j] = 1, e[j] = ~0ull;
+  for (;;) {
+    bool live = false;
+#pragma unroll
+    for (int j = 0; j < kSlots; ++j) {
+      // the next value of this slot that passes the first 32 primes
+      for (;;) {
+        if (k[j] == 0) {
+          e[j] = next;
+          if (next >= count) {  // no point left: the slot idles (s = 1 has no divisor)
+            e[j] = ~0ull;
+            s[j] = r[j] = 1;
+            break;
+          }
+          next += nw;
+          k[j] = 1;
+        }
+        const uint64_t n = pts[e[j]];
+        if (n < 3 || !(n & 1ull)) {
+          if (lane == 0) out[e[j]] = 0;
+          k[j] = 0;
+          continue;
+        }
+        if (k[j] >= 63 || (1ull << k[j]) >= n) {
+          if (lane == 0) out[e[j]] = kFailK;
+          k[j] = 0;
+          continue;
+        }
+        s[j] = n - (1ull << k[j]);
+        const uint64_t t = s[j] * small_inv;
+        const bool div = small_p && t <= small_lim;
+        if (__any_sync(0xFFFFFFFFu, div && t * small_inv <= small_lim)) {
+          ++k[j];
+          continue;
+        }
+        uint32_t m = __ballot_sync(0xFFFFFFFFu, div);
+        r[j] = s[j];
+        while (m) {
+          const int src = __ffs(m) - 1;
+          m &= m - 1;
+          r[j] *= __shfl_sync(0xFFFFFFFFu, small_inv, src);
+        }
+        live = true;
+        break;
+      }
+    }
+    if (!live) return;
+    uint64_t top = 0;
+#pragma unroll
+    for (int j = 0; j < kSlots; ++j) top = s[j] > top ? s[j] : top;
+    uint32_t bad = 0;
+    for (uint32_t base = 32; base < pt.n_div; base += 64) {
+      const uint64_t pb = pt.p[base];
+      if (pb * pb * pb > top) break;
+      uint64_t inv[2];
+      uint32_t lh[2];
+      bool any = false;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t i = base + 32u * u + lane;
+        inv[u] = i < pt.n_div ? pt.inv[i] : 0ull;  // (0 divides nothing: t = 0 is ruled out below)
+        lh[u] = i < pt.n_div ? lim_high(pt, i) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < kSlots; ++j) any |= maybe_divides(s[j], inv[u], lh[u]);
+      if (__any_sync(0xFFFFFFFFu, any)) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const uint32_t i = base + 32u * u + lane;
+          const uint64_t lim = i < pt.n_div ? pt.lim[i] : 0ull;
+#pragma unroll
+          for (int j = 0; j < kSlots; ++j) {
+            const uint64_t t = s[j] * inv[u];
+            const bool div = i < pt.n_div && t <= lim;
+            uint32_t m = __ballot_sync(0xFFFFFFFFu, div);
+            if (!m) continue;
+            if (__any_sync(0xFFFFFFFFu, div && t * inv[u] <= lim)) bad |= 1u << j;
+            while (m) {
+              const int src = __ffs(m) - 1;
+              m &= m - 1;
+              r[j] *= __shfl_sync(0xFFFFFFFFu, inv[u], src);
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kSlots; ++j) {
+      if (e[j] == ~0ull) continue;
+      if (!((bad >> j) & 1u) && cofactor_squarefree(r[j])) {
+        if (lane == 0) out[e[j]] = (uint8_t)k[j];
+        k[j] = 0;
+      } else {
+        ++k[j];
+      }
+    }
+  }
+}
+
+// Bound: few points by the latency of one pass over the primes (about 10^4 for
+// n near 2^50, ten per thread of a block), many by the multiplies (three per
+// prime and value).  One warp per point, with two 64-bit products, 64-bit
+// compares and two votes per 32 primes, took 143 us a call for one point (now
+// 30), 170 for 1024 (48) and 962 for 65536 on the device (372; with the whole
+// 64-bit product instead of its high word 396).
+// The lines: a block of 1024 threads per point while two fit every SM; smaller
+// blocks while a wave or two of them covers the points; then, with a thousand
+// points per SM's warps, the loads shared by four points.
+cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t num_sms,
                           cudaStream_t st) {
   if (count == 0) return cudaSuccess;
-  points_kernel<<<grid, 256, 0, st>>>(pt, pts, count, out);
+  const uint64_t sms = num_sms;
+  if (count <= 2 * sms)
+    points_block_kernel<4><<<(uint32_t)count, 1024, 0, st>>>(pt, pts, count, out);
+  else if (count <= 24 * sms)
+    points_block_kernel<2><<<(uint32_t)count, 256, 0, st>>>(pt, pts, count, out);
+  else
+    points_warp_kernel<<<(uint32_t)std::min<uint64_t>((count + 8 * kSlots - 1) / (8 * kSlots), 4 * sms), 256, 0, st>>>(
+        pt, pts, count, out);
   return cudaGetLastError();
 }
 

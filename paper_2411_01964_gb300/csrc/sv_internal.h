@@ -272,8 +272,8 @@ size_t stream_static_smem();
 cudaError_t stream_kernel_setup(int optin);
 cudaError_t launch_stream_tiles(const StreamArgs &s, uint32_t grid, cudaStream_t st);
 cudaError_t launch_stragglers(const StragArgs &a, uint32_t grid, cudaStream_t st);
-cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out,
-                          uint32_t grid, cudaStream_t st);
+cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t num_sms,
+                          cudaStream_t st);
 uint64_t host_isqrt(uint64_t x);  // floor(sqrt(x)), exact (host)
 cudaError_t build_prime_table(uint64_t pmax, uint32_t **d_p, uint64_t **d_mu, uint64_t **d_inv,
                               uint64_t **d_lim, uint32_t **d_bits, uint64_t *bits_words, uint32_t *n,
