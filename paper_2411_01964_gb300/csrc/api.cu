@@ -76,6 +76,7 @@ uint64_t range_odd_count(uint64_t lo, uint64_t hi) {
 namespace {
 
 constexpr uint64_t kMaxHi = 1ull << 62;
+constexpr uint32_t kLinearMinThreads = 256;  // threads per block of halved linear tiles
 
 sv_status cuda_status(cudaError_t e) { return e == cudaSuccess ? SV_OK : SV_ECUDA; }
 
@@ -152,14 +153,15 @@ uint64_t max_span_bits(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
 // single ranges of 2^34 and 2^36 integers: a sparse prime costs every tile
 // some work, a bucketed one only the tiles it strikes).
 // stream_threads: block size of the stream layout (streams.cu), 0 for the
-// linear one (tiles.cu).
-Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges = 0, uint32_t stream_threads = 0) {
+// linear one (tiles.cu), whose tiles `shrink` halves (see linear_shrink).
+Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges = 0, uint32_t stream_threads = 0,
+                       uint32_t shrink = 0) {
   const sv_config &k = c->cfg;
   Geometry g{};
-  g.tw = 1u << (k.tile_log2 - 5);
+  g.tw = 1u << (k.tile_log2 - shrink - 5);
   g.mw = 1u << (k.margin_log2 - 6);
-  g.threads = k.threads;
-  g.ctas = k.ctas_per_sm;
+  g.threads = std::max(k.threads >> shrink, std::min(k.threads, kLinearMinThreads));
+  g.ctas = std::min(k.ctas_per_sm * (k.threads / g.threads), std::max(k.ctas_per_sm, 4u));
   if (stream_threads) {
     g.stream = 1;
     g.threads = stream_threads;
@@ -248,9 +250,26 @@ uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, co
   return S;
 }
 
+// How often a launch of the linear layout halves its tiles: until there are
+// two tiles per SM, or a tile holds 2^15 odd n, or its margin is an eighth of
+// it.  (2^24 integers are 16 tiles of 2^19 odd n, which leave 136 SMs idle: with
+// the per-n output 643 us a call, 306 in 256 tiles.)
+uint32_t linear_shrink(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
+  const sv_config &k = c->cfg;
+  uint64_t bits = 0;
+  for (const RangeSpec &s : specs)
+    if (s.hi > s.lo) bits += (s.hi - s.lo) / 2;
+  uint32_t n = 0;
+  while (k.tile_log2 - n > 15 && k.margin_log2 - 1 + 3 < k.tile_log2 - n &&
+         specs.size() + (bits >> (k.tile_log2 - n)) < 2ull * (uint64_t)c->num_sms)
+    ++n;
+  return n;
+}
+
 // The geometry of one launch, with the bucket depth earlier launches grew to.
 Geometry geometry_of(const sv_ctx *c, const std::vector<RangeSpec> &specs, const Workspace &ws) {
-  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size(), stream_threads(c, specs, ws));
+  const uint32_t st = stream_threads(c, specs, ws);
+  Geometry g = make_geometry(c, max_span_bits(c, specs), specs.size(), st, st ? 0u : linear_shrink(c, specs));
   if (ws.bucket_cap > g.bucket_cap) g.bucket_cap = ws.bucket_cap;
   return g;
 }

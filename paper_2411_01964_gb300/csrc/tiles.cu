@@ -329,36 +329,6 @@ __device__ __noinline__ void straggler_push(const TileArgs &a, ScanShared &sh, u
   }
 }
 
-// Write the per-n minimal k of one word (bit-sliced planes pl[0..5]).
-__device__ __forceinline__ void write_per_n(uint8_t *out, uint64_t J0, uint64_t jlo, uint32_t valid,
-                                            const uint32_t pl[6]) {
-  while (valid) {
-    const uint32_t b = __ffs(valid) - 1;
-    valid &= valid - 1;
-    uint32_t k = 0;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) k |= ((pl[j] >> b) & 1u) << j;
-    out[J0 + b - jlo] = (uint8_t)k;
-  }
-}
-
-// One step of the word-parallel Algorithm 2 for k <= 5 (sf = flags of n - 2^k).
-//   LEAN: k = 1 is not counted (derived at the end of the tile from the
-//         number of valid n) and lists start at k >= 6 (T >= 6).
-template <int K, bool LEAN, bool PER_N>
-__device__ __forceinline__ void scan_step(uint32_t sf, uint32_t &unres, uint32_t &cnt, uint32_t pl[6],
-                                          const TileArgs &a, ScanShared &sh, int64_t aw, uint32_t rec_t) {
-  const uint32_t hit = unres & sf;
-  unres &= ~sf;
-  if (!(LEAN && K == 1)) cnt += __popc(hit);
-  if (PER_N) {
-#pragma unroll
-    for (int j = 0; j < 6; ++j)
-      if ((K >> j) & 1) pl[j] |= hit;
-  }
-  if (!LEAN && (uint32_t)K >= rec_t && hit) list_append(a, sh.req, hit, 32ull * (uint64_t)aw, (uint32_t)K);
-}
-
 // Mode 0: list entries (n with mink = k >= T) go to the tile's shared
 // buffer, which the tile's flush stages for the ordered list.  Entries
 // beyond the buffer are only counted; the flush reports them (kStListStage)
@@ -377,20 +347,14 @@ __device__ __noinline__ void list_buffer(ScanShared &sh, uint32_t hit, uint64_t 
 
 // k = 6 .. kwin (rare): whole-word look-back reads; counts, first occurrences
 // below T and lists go straight to shared/global atomics.
-template <bool LEAN, bool PER_N>
-__device__ __noinline__ uint32_t scan_tail(const uint32_t *win, uint32_t i, bool act, uint32_t unres,
-                                           uint32_t pl[6], const TileArgs &a, ScanShared &sh, int64_t aw,
-                                           uint32_t kwin, uint32_t rec_t) {
+template <bool LEAN>
+__device__ __noinline__ void scan_tail(const uint32_t *win, uint32_t i, bool act, uint32_t unres, const TileArgs &a,
+                                       ScanShared &sh, int64_t aw, uint32_t kwin, uint32_t rec_t) {
   const uint64_t J0 = 32ull * (uint64_t)aw;
   for (uint32_t k = 6; k <= kwin && __any_sync(0xFFFFFFFFu, unres); ++k) {
     const uint32_t sf = act ? win[i - (1u << (k - 6))] : 0u;
     const uint32_t hit = unres & sf;
     unres &= ~sf;
-    if (PER_N) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j)
-        if ((k >> j) & 1u) pl[j] |= hit;
-    }
     if (hit) {
       atomicAdd(&sh.hist[k], (unsigned long long)__popc(hit));
       if (LEAN || k < rec_t)
@@ -402,19 +366,18 @@ __device__ __noinline__ uint32_t scan_tail(const uint32_t *win, uint32_t i, bool
     }
   }
   if (unres) straggler_push(a, sh, unres, J0, kwin + 1u);
-  return unres;
 }
 
 // Record, for each k with a bit in `need`, the warp's first n with mink = k.
 // need is warp-uniform; a warp visits its words in increasing order, so its
 // first hit for k is its smallest, and the minimum over warps is the tile's.
 template <int K>
-__device__ __forceinline__ void record_first(uint32_t hit, uint32_t &need, ScanShared &sh, int64_t aw) {
+__device__ __forceinline__ void record_first(uint32_t hit, uint32_t &need, ScanShared &sh, uint64_t J0) {
   if (need & (1u << K)) {
     const uint32_t bal = __ballot_sync(0xFFFFFFFFu, hit != 0);
     if (bal) {
       if ((threadIdx.x & 31u) == (uint32_t)(__ffs(bal) - 1))
-        atomicMin(&sh.first[K], (unsigned long long)(64ull * (uint64_t)aw + 2ull * (uint64_t)(__ffs(hit) - 1) + 1ull));
+        atomicMin(&sh.first[K], (unsigned long long)(2ull * (J0 + (uint64_t)(__ffs(hit) - 1)) + 1ull));
       need &= ~(1u << K);
     }
   }
@@ -422,7 +385,7 @@ __device__ __forceinline__ void record_first(uint32_t hit, uint32_t &need, ScanS
 
 // One warp-iteration of the scan: lane's word i.  REC: some of the frequent
 // exponents (k <= 5) still lack this warp's first occurrence.
-template <bool LEAN, bool PER_N, bool REC>
+template <bool LEAN, bool REC>
 __device__ __forceinline__ void scan_word(const uint32_t *win, uint32_t i, bool act, int64_t aw, uint32_t valid,
                                           uint32_t &need, uint32_t &c1, uint32_t &c2, uint32_t &c3, uint32_t &c4,
                                           uint32_t &c5, const TileArgs &a, ScanShared &sh) {
@@ -430,16 +393,12 @@ __device__ __forceinline__ void scan_word(const uint32_t *win, uint32_t i, bool 
   const uint32_t w = act ? win[i] : 0u;
   const uint32_t wp = act ? win[i - 1] : 0u;
   uint32_t unres = valid;
-  uint32_t pl[6] = {0u, 0u, 0u, 0u, 0u, 0u};
   uint32_t h;
 #define SV_STEP(K, SF, CNT)                                     \
   h = unres & (SF);                                             \
   unres &= ~(SF);                                               \
   if (!(LEAN && K == 1)) CNT += __popc(h);                      \
-  if (PER_N) {                                                  \
-    _Pragma("unroll") for (int j = 0; j < 6; ++j) if ((K >> j) & 1) pl[j] |= h; \
-  }                                                             \
-  if (REC) record_first<K>(h, need, sh, aw);                    \
+  if (REC) record_first<K>(h, need, sh, 32ull * (uint64_t)aw);                    \
   if (!LEAN && (uint32_t)K >= rec_t && h) list_append(a, sh.req, h, 32ull * (uint64_t)aw, (uint32_t)K);
   SV_STEP(1, __funnelshift_l(wp, w, 1), c1)
   if (__any_sync(0xFFFFFFFFu, unres)) {
@@ -450,13 +409,12 @@ __device__ __forceinline__ void scan_word(const uint32_t *win, uint32_t i, bool 
         SV_STEP(4, __funnelshift_l(wp, w, 8), c4)
         if (__any_sync(0xFFFFFFFFu, unres)) {
           SV_STEP(5, __funnelshift_l(wp, w, 16), c5)
-          if (__any_sync(0xFFFFFFFFu, unres)) scan_tail<LEAN, PER_N>(win, i, act, unres, pl, a, sh, aw, kwin, rec_t);
+          if (__any_sync(0xFFFFFFFFu, unres)) scan_tail<LEAN>(win, i, act, unres, a, sh, aw, kwin, rec_t);
         }
       }
     }
   }
 #undef SV_STEP
-  if (PER_N && sh.req.per_n_k) write_per_n(sh.req.per_n_k, 32ull * (uint64_t)aw, sh.req.jlo, valid, pl);
 }
 
 
@@ -562,8 +520,8 @@ __device__ __forceinline__ void scan_tile_lean(const uint32_t *win, const TileAr
     if (i1 - ifl < nfull) v1 = 0xFFFFFFFFu;
     else v1 = a1 ? valid_mask(32ull * (uint64_t)aw1, sh.req.jlo, sh.req.jhi) : 0u;
     if (need) {
-      scan_word<true, false, true>(win, i0, a0, aw0, v0, need, c1, c2, c3, c4, c5, a, sh);
-      scan_word<true, false, true>(win, i1, a1, aw1, v1, need, c1, c2, c3, c4, c5, a, sh);
+      scan_word<true, true>(win, i0, a0, aw0, v0, need, c1, c2, c3, c4, c5, a, sh);
+      scan_word<true, true>(win, i1, a1, aw1, v1, need, c1, c2, c3, c4, c5, a, sh);
       continue;
     }
     const uint32_t w0 = a0 ? win[i0] : 0u, p0 = a0 ? win[i0 - 1] : 0u;
@@ -601,7 +559,7 @@ __device__ __forceinline__ void scan_tile_lean(const uint32_t *win, const TileAr
   }
 }
 
-template <bool LEAN, bool PER_N>
+template <bool LEAN>
 __device__ __forceinline__ void scan_tile(const uint32_t *win, const TileArgs &a, ScanShared &sh, int64_t wstart,
                                           uint32_t nwords, uint32_t ifl, uint32_t nfull) {
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -617,9 +575,9 @@ __device__ __forceinline__ void scan_tile(const uint32_t *win, const TileArgs &a
     if (i - ifl < nfull) valid = 0xFFFFFFFFu;
     else valid = act ? valid_mask(32ull * (uint64_t)aw, sh.req.jlo, sh.req.jhi) : 0u;
     if (need)
-      scan_word<LEAN, PER_N, true>(win, i, act, aw, valid, need, c1, c2, c3, c4, c5, a, sh);
+      scan_word<LEAN, true>(win, i, act, aw, valid, need, c1, c2, c3, c4, c5, a, sh);
     else
-      scan_word<LEAN, PER_N, false>(win, i, act, aw, valid, need, c1, c2, c3, c4, c5, a, sh);
+      scan_word<LEAN, false>(win, i, act, aw, valid, need, c1, c2, c3, c4, c5, a, sh);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -635,6 +593,128 @@ __device__ __forceinline__ void scan_tile(const uint32_t *win, const TileArgs &a
     if (c3) atomicAdd(&sh.hist[3], (unsigned long long)c3);
     if (c4) atomicAdd(&sh.hist[4], (unsigned long long)c4);
     if (c5) atomicAdd(&sh.hist[5], (unsigned long long)c5);
+  }
+}
+
+// ---- the scan with the per-n output ------------------------------------------
+// One byte per n makes the output the path's traffic: 32 bytes per word of n.
+// Each lane takes the 32 n of one 32-byte group of the output (the groups are
+// aligned in memory, so their first bit lies anywhere in a window word) and
+// writes them with one 32-byte store, a warp 1 KB.  With u1, u2, u3 the n left
+// after k = 1, 2, 3 (each a part of the one before), k - 1 = 0..3 is the two-bit
+// code c0 = u1 ^ u2 ^ u3, c1 = u2; four n's codes index a table of their four
+// bytes: 29 instructions for 32 bytes, against about 12 per byte for setting
+// each from bit-sliced values.  The few n left after k = 4 (one word in 230
+// has any) are stored over it byte by byte.
+// 2^31 integers near 2^44 (1.07 GB of output): 363 us a call, 3 TB/s, against
+// 5770 us.
+
+// Entry i: the bytes of four n whose codes are bits 0-3 (c0) and 4-7 (c1) of i.
+__device__ __forceinline__ void build_per_n_lut(uint32_t *lut) {
+  for (uint32_t i = threadIdx.x; i < 256u; i += blockDim.x) {
+    uint32_t v = 0;
+    for (uint32_t n = 0; n < 4; ++n) v |= (1u + ((i >> n) & 1u) + 2u * ((i >> (4 + n)) & 1u)) << (8u * n);
+    lut[i] = v;
+  }
+}
+
+// The flags of the 32 bits from window bit P on; bits outside the window read
+// as 0 (only n outside the tile look there).
+__device__ __forceinline__ uint32_t window_bits(const uint32_t *win, int32_t P, uint32_t nwords) {
+  const int32_t i = P >> 5;
+  const uint32_t lo = (uint32_t)i < nwords ? win[i] : 0u, hi = (uint32_t)(i + 1) < nwords ? win[i + 1] : 0u;
+  return __funnelshift_r(lo, hi, (uint32_t)P & 31u);
+}
+
+// The n (bits u of the group at window bit P, output byte x) left after
+// k = 4: k = 5 .. kwin by look-back, then the exact test (which writes its own byte).
+__device__ __noinline__ void finish_per_n(const uint32_t *win, int32_t P, uint32_t nwords, uint32_t u, uint64_t J,
+                                          uint8_t *out, const TileArgs &a, ScanShared &sh) {
+  const uint32_t kwin = a.g.kwin, rec_t = a.g.rec_t;
+  for (uint32_t k = 5; k <= kwin && u; ++k) {
+    const uint32_t h = u & window_bits(win, P - (1 << (k - 1)), nwords);
+    u ^= h;
+    if (!h) continue;
+    atomicAdd(&sh.hist[k], (unsigned long long)__popc(h));
+    atomicMin(&sh.first[k], (unsigned long long)(2ull * (J + (uint64_t)(__ffs(h) - 1)) + 1ull));
+    if (k >= rec_t) list_append(a, sh.req, h, J, k);
+    for (uint32_t m = h; m; m &= m - 1) out[__ffs(m) - 1] = (uint8_t)k;
+  }
+  if (u) straggler_push(a, sh, u, J, kwin + 1u);
+}
+
+__device__ __forceinline__ void scan_tile_per_n(const uint32_t *win, const TileArgs &a, ScanShared &sh,
+                                                const uint32_t *lut, int64_t wstart, uint32_t nwords) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const ReqDesc &R = sh.req;
+  const uint32_t rec_t = a.g.rec_t;
+  uint8_t *const out = R.per_n_k;
+  // the tile's n as window bits [vl, vh), and the window bit of the 32-byte
+  // group that holds the first (window bit P is output byte P + xoff)
+  const int64_t wbit = 32 * wstart;
+  const int32_t vl = (int32_t)(max((int64_t)R.jlo, wbit + 32 * (int64_t)a.g.mw) - wbit);
+  const int32_t vh = (int32_t)(min((int64_t)R.jhi, wbit + 32 * (int64_t)nwords) - wbit);
+  const int64_t xoff = wbit - (int64_t)R.jlo;
+  const int32_t P0 = vl - (int32_t)(((uintptr_t)out + (uint64_t)(vl + xoff)) & 31u);  // > -32
+  uint32_t need = sh.need;
+  uint32_t U0 = 0, U1 = 0, U2 = 0, U3 = 0, U4 = 0;  // n in all, and left after k = 1 .. 4
+  for (int32_t Pw = P0 + 1024 * (int32_t)warp; Pw < vh; Pw += 1024 * (int32_t)nwarps) {
+    const int32_t P = Pw + 32 * (int32_t)lane;
+    uint32_t valid = 0xFFFFFFFFu;
+    if (P < vl) valid &= vl - P >= 32 ? 0u : 0xFFFFFFFFu << (vl - P);
+    if (P + 32 > vh) valid &= P >= vh ? 0u : 0xFFFFFFFFu >> (P + 32 - vh);
+    const uint32_t X = window_bits(win, P, nwords), Y = window_bits(win, P - 32, nwords);
+    const uint32_t u1 = valid & ~__funnelshift_l(Y, X, 1);
+    const uint32_t u2 = u1 & ~__funnelshift_l(Y, X, 2);
+    const uint32_t u3 = u2 & ~__funnelshift_l(Y, X, 4);
+    const uint32_t u4 = u3 & ~__funnelshift_l(Y, X, 8);
+    U0 += __popc(valid);
+    U1 += __popc(u1);
+    U2 += __popc(u2);
+    U3 += __popc(u3);
+    U4 += __popc(u4);
+    const uint64_t J = (uint64_t)(wbit + (int64_t)P);
+    const uint32_t c0 = u1 ^ u2 ^ u3, c1 = u2;
+    uint8_t *const o = out + (P + xoff);
+    if (valid == 0xFFFFFFFFu) {
+      // byte j of ev / od: the table index of the n 8j .. 8j + 3 / 8j + 4 .. 8j + 7
+      const uint32_t ev = (c0 & 0x0F0F0F0Fu) | ((c1 & 0x0F0F0F0Fu) << 4);
+      const uint32_t od = ((c0 >> 4) & 0x0F0F0F0Fu) | (c1 & 0xF0F0F0F0u);
+      uint32_t v[8];
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) {
+        v[2 * j] = lut[(ev >> (8 * j)) & 0xFFu];
+        v[2 * j + 1] = lut[(od >> (8 * j)) & 0xFFu];
+      }
+      asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                   "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                   : "memory");
+    } else {
+      for (uint32_t m = valid & ~u4; m; m &= m - 1) {
+        const uint32_t b = __ffs(m) - 1;
+        o[b] = (uint8_t)(1u + ((c0 >> b) & 1u) + 2u * ((c1 >> b) & 1u));
+      }
+    }
+    if (need) {  // a first occurrence of k <= 4 may be here
+      record_first<1>(valid & ~u1, need, sh, J);
+      record_first<2>(u1 & ~u2, need, sh, J);
+      record_first<3>(u2 & ~u3, need, sh, J);
+      record_first<4>(u3 & ~u4, need, sh, J);
+    }
+    if (rec_t <= 4) {
+      if (rec_t <= 1 && (valid & ~u1)) list_append(a, R, valid & ~u1, J, 1);
+      if (rec_t <= 2 && (u1 & ~u2)) list_append(a, R, u1 & ~u2, J, 2);
+      if (rec_t <= 3 && (u2 & ~u3)) list_append(a, R, u2 & ~u3, J, 3);
+      if (u3 & ~u4) list_append(a, R, u3 & ~u4, J, 4);
+    }
+    if (u4) finish_per_n(win, P, nwords, u4, J, o, a, sh);
+    __syncwarp();
+  }
+  const uint32_t h[5] = {0, U0 - U1, U1 - U2, U2 - U3, U3 - U4};  // (k >= 5: counted one by one)
+#pragma unroll
+  for (int k = 1; k <= 4; ++k) {
+    const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, h[k]);
+    if (lane == 0 && c) atomicAdd(&sh.hist[k], (unsigned long long)c);
   }
 }
 
@@ -672,6 +752,7 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
   __shared__ uint32_t stab[StampTab<NS>::kSize];
   constexpr bool LEAN = (MODE == 0);
   constexpr bool PER_N = (MODE == 2);
+  __shared__ uint32_t lut[PER_N ? 256 : 1];
 
   const uint32_t tid = threadIdx.x, S = blockDim.x;
   const uint32_t lane = tid & 31u, warp = tid >> 5;
@@ -693,6 +774,7 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
   uint32_t load_parity = 0;     // phase parity of the next bulk window load
   bool store_pending = false;   // thread 0: a bulk store may still read the window
   build_stamp_tables<NS>(stab);
+  if (PER_N) build_per_n_lut(lut);
   const uint32_t T = 32u * g.tw;  // a window starts T bits above the previous one
   if (tid == 0) {
     sh.n_strag = 0;
@@ -974,8 +1056,10 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
       const uint32_t nfull = fh > fl ? (uint32_t)(fh - fl) : 0u;
       if (LEAN)
         scan_tile_lean(win, a, sh, wstart, nwords, ifl, nfull);
+      else if (PER_N && R.per_n_k)
+        scan_tile_per_n(win, a, sh, lut, wstart, nwords);
       else
-        scan_tile<LEAN, PER_N>(win, a, sh, wstart, nwords, ifl, nfull);
+        scan_tile<LEAN>(win, a, sh, wstart, nwords, ifl, nfull);
     }
     if (tid == 0) {
       sh.next_tile = next;
