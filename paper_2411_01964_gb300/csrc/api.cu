@@ -20,22 +20,17 @@ namespace sv {
 std::atomic<uint32_t> g_inject_alloc_failures{0};
 
 void Workspace::release_all() {
-  if (gexec) cudaGraphExecDestroy(gexec);
-  gexec = nullptr;
-  if (graph) cudaGraphDestroy(graph);
-  graph = nullptr;
-  for (cudaEvent_t &e : gev) {
-    if (e) cudaEventDestroy(e);
-    e = nullptr;
+  for (LaunchGraph &lg : graphs) {
+    if (lg.exec) cudaGraphExecDestroy(lg.exec);
+    if (lg.graph) cudaGraphDestroy(lg.graph);
+    for (cudaEvent_t &e : lg.ev)
+      if (e) cudaEventDestroy(e);
+    lg = LaunchGraph{};
   }
   if (staged) cudaEventDestroy(staged);
   staged = nullptr;
-  reqs.release();
-  h_reqs.release();
-  hdr.release();
-  h_hdr.release();
-  slots.release();
-  h_slots.release();
+  io.release();
+  h_io.release();
   list_n.release();
   list_k.release();
   h_list_n.release();
@@ -187,6 +182,9 @@ Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges 
   uint64_t lp = k.large_prime_min;
   if (span_bits) {
     uint64_t lp_span = host_isqrt(span_bits / 64) + 1;
+    uint64_t lp2 = 1;  // a power of two: launches of similar ranges share a geometry, and with it a captured graph
+    while (lp2 < lp_span) lp2 *= 2;
+    lp_span = lp2;
     if (n_ranges && n_ranges <= kFillReqChunk) lp_span = std::min(lp_span, kSegmentedLargeMin);
     lp = std::max<uint64_t>(lp, lp_span);
   }
@@ -318,13 +316,54 @@ sv_status ensure_tile_smem(sv_ctx *c) {
   return SV_OK;
 }
 
+// Ranges a launch's buffers are laid out for: exactly n of few, else a power
+// of two (so that launches of similar sizes share a captured graph).
+uint32_t range_class(uint32_t n) {
+  if (n <= kHostPlanMax) return n ? n : 1;
+  uint32_t m = 2 * kHostPlanMax;
+  while (m < n) m *= 2;
+  return m;
+}
+
+// Lays out the exchange block for n ranges with list_total list entries.
+// Short lists lie behind the slots and come back with them in one copy; 4096
+// entries take 36 KB, about as long as a second copy takes to start.
+constexpr uint64_t kShortLists = 4096;
+sv_status layout_io(Workspace &ws, uint32_t n, uint64_t list_total) {
+  const size_t m = range_class(n);
+  ws.io_hdr = (sizeof(ReqDesc) * m + 255) & ~(size_t)255;
+  ws.io_slots = ws.io_hdr + ((sizeof(LaunchHeader) + 63) & ~(size_t)63);
+  ws.io_list = ws.io_slots + sizeof(ResultSlot) * m;
+  ws.io_end = ws.io_list;
+  uint64_t room = 0;
+  if (list_total <= kShortLists) {
+    room = 64;
+    while (room < list_total) room *= 2;
+    ws.io_end += 9 * room;
+  }
+  if (ws.io.ensure(ws.io_end) || ws.h_io.ensure(ws.io_end)) return SV_ENOMEM;
+  if (!room && (ws.list_n.ensure(list_total) || ws.list_k.ensure(list_total))) return SV_ENOMEM;
+  unsigned char *d = ws.io.p, *h = ws.h_io.p;
+  ws.reqs = (ReqDesc *)d;
+  ws.h_reqs = (ReqDesc *)h;
+  ws.hdr = (LaunchHeader *)(d + ws.io_hdr);
+  ws.h_hdr = (LaunchHeader *)(h + ws.io_hdr);
+  ws.slots = (ResultSlot *)(d + ws.io_slots);
+  ws.h_slots = (ResultSlot *)(h + ws.io_slots);
+  ws.d_list_n = room ? (uint64_t *)(d + ws.io_list) : ws.list_n.p;
+  ws.d_list_k = room ? d + ws.io_list + 8 * room : ws.list_k.p;
+  return SV_OK;
+}
+
 // Plans the descriptors of `specs` into ws.h_reqs / ws.h_hdr.
 sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g, Workspace &ws) {
   const uint32_t n = (uint32_t)specs.size();
   // the previous launch may still be copying from the pinned staging
   if (ws.staged && cudaEventSynchronize(ws.staged) != cudaSuccess) return SV_ECUDA;
-  if (ws.h_reqs.ensure(n ? n : 1) != cudaSuccess) return SV_ENOMEM;
-  if (ws.h_hdr.ensure(1) != cudaSuccess) return SV_ENOMEM;
+  uint64_t all_lists = 0;
+  for (const RangeSpec &s : specs) all_lists += s.list_cap;
+  const sv_status ls = layout_io(ws, n, all_lists);
+  if (ls) return ls;
   uint64_t tiles = 0, list_total = 0, fail_total = 0;
   uint32_t max_primes = 0;
   uint64_t jhi_max = 0;  // the largest odd multiplier floor((2 jhi - 1) / p_hyb^2) grows with jhi
@@ -382,7 +421,12 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
     d.bitmap_in = s.bitmap_in;
     d.bitmap_w0 = s.bitmap_w0;
     all_from_bitmap &= (s.bitmap_in != nullptr);
-    ws.h_reqs.p[r] = d;
+    ws.h_reqs[r] = d;
+    if (n <= kHostPlanMax) {  // the result slot as the launch finds it (many ranges: by the init kernel)
+      ResultSlot &slot = ws.h_slots[r];
+      std::memset(&slot, 0, sizeof(slot));
+      for (int k = 0; k < kMaxK; ++k) slot.first_n[k] = kNoN;
+    }
   }
   if (hi_max > 1) max_primes = primes_upto(c, host_isqrt(hi_max - 1));
   LaunchHeader h{};
@@ -396,7 +440,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
   h.n_reqs = n;
   h.total_tiles = (uint32_t)tiles;
   h.max_primes = max_primes;
-  *ws.h_hdr.p = h;
+  *ws.h_hdr = h;
   ws.n_reqs = n;
   ws.total_tiles = (uint32_t)tiles;
   ws.max_primes = max_primes;
@@ -417,6 +461,87 @@ int launch_mode(const Workspace &ws) { return ws.any_per_n ? 2 : (ws.ordered ? 0
 bool ensure_stage(Workspace &ws) {
   const size_t t = ws.total_tiles ? ws.total_tiles : 1;
   return !(ws.stage_n.ensure(t * kStageCap) || ws.stage_k.ensure(t * kStageCap) || ws.stage_cnt.ensure(t));
+}
+
+// The device buffers of the planned launch.
+sv_status ensure_buffers(Workspace &ws, const Geometry &g, int mode) {
+  const size_t tiles = ws.total_tiles ? ws.total_tiles : 1;
+  const size_t counts = ws.bucket_count.cap;
+  if (ws.fail_n.ensure(ws.fail_total ? ws.fail_total : 1) || ws.strag.ensure(ws.strag_cap) ||
+      ws.bucket_count.ensure(tiles) || ws.bucket_data.ensure(tiles * g.bucket_cap))
+    return SV_ENOMEM;
+  if (ws.bucket_count.cap != counts) ws.counts_clean = false;  // grown (perhaps in place)
+  if (mode == 0 && !ensure_stage(ws)) return SV_ENOMEM;
+  return SV_OK;
+}
+
+// What the straggler and compaction kernels of the planned launch take.
+void finish_args(const sv_ctx *c, const Geometry &g, Workspace &ws, int mode) {
+  StragArgs &s = ws.strag_args;
+  s = StragArgs{};
+  s.pt = prime_tab(c);
+  s.reqs = ws.reqs;
+  s.hdr = ws.hdr;
+  s.slots = ws.slots;
+  s.list_n = ws.d_list_n;
+  s.list_k = ws.d_list_k;
+  s.fail_n = ws.fail_n.p;
+  s.strag = ws.strag.p;
+  s.strag_cap = ws.strag_cap;
+  s.rec_t = g.rec_t;
+  ws.compact_grid = 0;
+  if (mode != 0) return;
+  s.stage_n = ws.stage_n.p;
+  s.stage_k = ws.stage_k.p;
+  s.stage_cnt = ws.stage_cnt.p;
+  s.stage_cap = g.stage_cap;
+  s.tw = g.tw;
+  s.tw_inv = g.tw_inv;
+  CompactArgs &ca = ws.compact_args;
+  ca = CompactArgs{};
+  ca.reqs = ws.reqs;
+  ca.hdr = ws.hdr;
+  ca.slots = ws.slots;
+  ca.list_n = ws.d_list_n;
+  ca.list_k = ws.d_list_k;
+  ca.stage_n = ws.stage_n.p;
+  ca.stage_k = ws.stage_k.p;
+  ca.stage_cnt = ws.stage_cnt.p;
+  ca.stage_cap = g.stage_cap;
+  ws.compact_grid = std::min<uint32_t>((ws.total_tiles + 127) / 128, 4u * (uint32_t)c->num_sms);
+}
+
+// The arguments of the fill and tile kernels of the planned launch.
+TileArgs tile_args(const sv_ctx *c, const Geometry &g, const Workspace &ws, int mode) {
+  TileArgs t{};
+  t.pt = prime_tab(c);
+  t.g = g;
+  t.reqs = ws.reqs;
+  t.hdr = ws.hdr;
+  t.slots = ws.slots;
+  t.list_n = ws.d_list_n;
+  t.list_k = ws.d_list_k;
+  t.fail_n = ws.fail_n.p;
+  t.strag = ws.strag.p;
+  t.strag_cap = ws.strag_cap;
+  t.bucket_count = ws.bucket_count.p;
+  t.bucket_data = ws.bucket_data.p;
+  if (mode == 0) {
+    t.stage_n = ws.stage_n.p;
+    t.stage_k = ws.stage_k.p;
+    t.stage_cnt = ws.stage_cnt.p;
+  }
+  return t;
+}
+BucketArgs bucket_args(const sv_ctx *c, const Geometry &g, const Workspace &ws) {
+  BucketArgs b{};
+  b.pt = prime_tab(c);
+  b.g = g;
+  b.reqs = ws.reqs;
+  b.hdr = ws.hdr;
+  b.bucket_count = ws.bucket_count.p;
+  b.bucket_data = ws.bucket_data.p;
+  return b;
 }
 
 // Blocks of the bucket fill: one full wave.
@@ -461,104 +586,47 @@ struct KTimer {
 // Enqueues init -> bucket fill -> tiles -> stragglers for the planned launch.
 sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) {
   const uint32_t n = ws.n_reqs;
-  if (ws.reqs.ensure(n ? n : 1) || ws.hdr.ensure(1) || ws.slots.ensure(n ? n : 1) ||
-      ws.h_slots.ensure(n ? n : 1) || ws.list_n.ensure(ws.list_total ? ws.list_total : 1) ||
-      ws.list_k.ensure(ws.list_total ? ws.list_total : 1) || ws.fail_n.ensure(ws.fail_total ? ws.fail_total : 1) ||
-      ws.strag.ensure(ws.strag_cap) || ws.bucket_count.ensure(ws.total_tiles ? ws.total_tiles : 1) ||
-      ws.bucket_data.ensure((size_t)(ws.total_tiles ? ws.total_tiles : 1) * g.bucket_cap))
-    return SV_ENOMEM;
   const int mode = launch_mode(ws);
-  if (mode == 0 && !ensure_stage(ws)) return SV_ENOMEM;
+  const sv_status bs = ensure_buffers(ws, g, mode);
+  if (bs) return bs;
   ws.bucket_cap = g.bucket_cap;
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.reqs.p, ws.h_reqs.p, sizeof(ReqDesc) * n, cudaMemcpyHostToDevice, st));
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.hdr.p, ws.h_hdr.p, sizeof(LaunchHeader), cudaMemcpyHostToDevice, st));
-  ws.h2d_bytes = sizeof(ReqDesc) * n + sizeof(LaunchHeader);
+  const size_t in_bytes = ws.io_slots;  // descriptors and header (the init kernel sets the slots)
+  SV_TRY_CUDA(cudaMemcpyAsync(ws.io.p, ws.h_io.p, in_bytes, cudaMemcpyHostToDevice, st));
+  ws.h2d_bytes = in_bytes;
   if (!ws.staged && cudaEventCreateWithFlags(&ws.staged, cudaEventDisableTiming) != cudaSuccess) return SV_ECUDA;
   SV_TRY_CUDA(cudaEventRecord(ws.staged, st));
   {
     KTimer kt(c, kKInit, st);
-    SV_TRY_CUDA(launch_init(ws.hdr.p, ws.slots.p, n, ws.bucket_count.p, mode == 0 ? ws.stage_cnt.p : nullptr,
-                            ws.total_tiles, ws.reqs.p, g.mw, c->d_p, c->n_primes, p_hyb_sq(g), st));
+    SV_TRY_CUDA(launch_init(ws.hdr, ws.slots, n, ws.bucket_count.p, mode == 0 ? ws.stage_cnt.p : nullptr,
+                            ws.total_tiles, ws.reqs, g.mw, c->d_p, c->n_primes, p_hyb_sq(g), st));
     kt.done();
   }
   c->launches++;
-  const PrimeTab pt = prime_tab(c);
+  ws.lazy_strag = false;
+  ws.counts_clean = false;  // (a launch of a bitmap's windows leaves the counts alone)
   if (ws.max_primes > g.i_large && ws.total_tiles && !ws.all_from_bitmap) {
-    BucketArgs b{};
-    b.pt = pt;
-    b.g = g;
-    b.reqs = ws.reqs.p;
-    b.hdr = ws.hdr.p;
-    b.bucket_count = ws.bucket_count.p;
-    b.bucket_data = ws.bucket_data.p;
     KTimer kt(c, kKBucket, st);
-    SV_TRY_CUDA(launch_bucket_fill(b, ws.max_primes - g.i_large, n, ws.j_max, fill_blocks(c), st));
+    SV_TRY_CUDA(launch_bucket_fill(bucket_args(c, g, ws), ws.max_primes - g.i_large, n, ws.j_max, fill_blocks(c), st));
     kt.done();
     c->launches++;
   }
   if (ws.total_tiles) {
-    TileArgs t{};
-    t.pt = pt;
-    t.g = g;
-    t.reqs = ws.reqs.p;
-    t.hdr = ws.hdr.p;
-    t.slots = ws.slots.p;
-    t.list_n = ws.list_n.p;
-    t.list_k = ws.list_k.p;
-    t.fail_n = ws.fail_n.p;
-    t.strag = ws.strag.p;
-    t.strag_cap = ws.strag_cap;
-    t.bucket_count = ws.bucket_count.p;
-    t.bucket_data = ws.bucket_data.p;
-    if (mode == 0) {
-      t.stage_n = ws.stage_n.p;
-      t.stage_k = ws.stage_k.p;
-      t.stage_cnt = ws.stage_cnt.p;
-    }
     {
       KTimer kt(c, ws.tile_kernel_id, st);
-      SV_TRY_CUDA(launch_tile_stage(c, t, mode, ws.search_all, ws.total_tiles, st));
+      SV_TRY_CUDA(launch_tile_stage(c, tile_args(c, g, ws, mode), mode, ws.search_all, ws.total_tiles, st));
       kt.done();
     }
     c->launches++;
-    StragArgs s{};
-    s.pt = pt;
-    s.reqs = ws.reqs.p;
-    s.hdr = ws.hdr.p;
-    s.slots = ws.slots.p;
-    s.list_n = ws.list_n.p;
-    s.list_k = ws.list_k.p;
-    s.fail_n = ws.fail_n.p;
-    s.strag = ws.strag.p;
-    s.strag_cap = ws.strag_cap;
-    s.rec_t = g.rec_t;
-    if (mode == 0) {
-      s.stage_n = ws.stage_n.p;
-      s.stage_k = ws.stage_k.p;
-      s.stage_cnt = ws.stage_cnt.p;
-      s.stage_cap = g.stage_cap;
-      s.tw = g.tw;
-      s.tw_inv = g.tw_inv;
-    }
+    finish_args(c, g, ws, mode);
     {
       KTimer kt(c, kKStrag, st);
-      SV_TRY_CUDA(launch_stragglers(s, (uint32_t)c->num_sms * 2, st));
+      SV_TRY_CUDA(launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st));
       kt.done();
     }
     c->launches++;
-    if (mode == 0) {
-      CompactArgs ca{};
-      ca.reqs = ws.reqs.p;
-      ca.hdr = ws.hdr.p;
-      ca.slots = ws.slots.p;
-      ca.list_n = ws.list_n.p;
-      ca.list_k = ws.list_k.p;
-      ca.stage_n = ws.stage_n.p;
-      ca.stage_k = ws.stage_k.p;
-      ca.stage_cnt = ws.stage_cnt.p;
-      ca.stage_cap = g.stage_cap;
+    if (ws.compact_grid) {
       KTimer kt(c, kKCompact, st);
-      SV_TRY_CUDA(launch_compact(ca, std::min<uint32_t>((ws.total_tiles + 127) / 128, 4u * (uint32_t)c->num_sms), st));
+      SV_TRY_CUDA(launch_compact(ws.compact_args, ws.compact_grid, st));
       kt.done();
       c->launches++;
     }
@@ -567,122 +635,70 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
 }
 
 // The same launch as a CUDA graph.  The grids are fixed and persistent (every
-// kernel reads the launch's sizes from the device header), so one captured
-// graph is replayed for every launch that fits the current buffers, geometry
-// and kernel mode; it is re-captured when any of them changes.
+// kernel reads the launch's sizes from the device header), so a captured graph
+// is replayed for every launch that fits the current buffers, geometry and
+// kernel mode; the workspace keeps the last kGraphs of them.
+// It is leaner than enqueue(): one copy in; no init kernel for few ranges
+// (their slots come with the copy, the bucket counts are left clear by the
+// previous launch); and no straggler kernel where the look-back reaches
+// k = 12, beyond which one odd n in 10^15 remains: the host runs that kernel
+// when the header counts a straggler (collect).  A launch with the per-n output
+// keeps it, its output may be read before the results are fetched.
 sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) {
   const uint32_t n = ws.n_reqs;
-  if (ws.reqs.ensure(n ? n : 1) || ws.hdr.ensure(1) || ws.slots.ensure(n ? n : 1) ||
-      ws.h_slots.ensure(n ? n : 1) || ws.list_n.ensure(ws.list_total ? ws.list_total : 1) ||
-      ws.list_k.ensure(ws.list_total ? ws.list_total : 1) || ws.fail_n.ensure(ws.fail_total ? ws.fail_total : 1) ||
-      ws.strag.ensure(ws.strag_cap) || ws.bucket_count.ensure(ws.total_tiles ? ws.total_tiles : 1) ||
-      ws.bucket_data.ensure((size_t)(ws.total_tiles ? ws.total_tiles : 1) * g.bucket_cap))
-    return SV_ENOMEM;
   const int mode = launch_mode(ws);
-  if (mode == 0 && !ensure_stage(ws)) return SV_ENOMEM;
+  const sv_status bs = ensure_buffers(ws, g, mode);
+  if (bs) return bs;
   ws.bucket_cap = g.bucket_cap;
-  const size_t req_copy = std::min(ws.h_reqs.cap, ws.reqs.cap);
+  const bool init = n > kHostPlanMax;
+  const size_t in_bytes = init ? ws.io_slots : ws.io_list;
+  ws.lazy_strag = g.kwin >= 12 && mode != 2;
   GraphKey key;
   std::memset(&key, 0, sizeof(key));
-  const void *ptrs[] = {ws.reqs.p,    ws.hdr.p,   ws.slots.p,        ws.list_n.p,       ws.list_k.p,
-                        ws.fail_n.p,  ws.strag.p, ws.bucket_count.p, ws.bucket_data.p, ws.h_reqs.p,
-                        ws.h_hdr.p,   c->d_p,     (const void *)st,  ws.stage_n.p,      ws.stage_k.p,
-                        ws.stage_cnt.p};
+  const void *ptrs[] = {ws.io.p,      ws.h_io.p,  ws.slots,          ws.d_list_n,        ws.d_list_k,
+                        ws.fail_n.p,  ws.strag.p, ws.bucket_count.p, ws.bucket_data.p,   c->d_p,
+                        (const void *)st, ws.stage_n.p, ws.stage_k.p, ws.stage_cnt.p};
+  static_assert(sizeof(ptrs) <= sizeof(key.p), "the key holds every pointer");
   std::memcpy(key.p, ptrs, sizeof(ptrs));
   key.g = g;
   key.mode = (uint32_t)mode;
   key.strag_cap = ws.strag_cap;
   key.search_all = ws.search_all ? 1u : 0u;
-  key.req_copy = req_copy;
+  key.n_class = range_class(n);
+  key.in_bytes = in_bytes;
   key.n_table = c->n_primes;
   // per-kernel timing of the tile kernel: event-record nodes around it
   const bool timed = ((c->kprof >> ws.tile_kernel_id) & 1u) && st == c->stream;
   key.timed = timed ? 1u : 0u;
-  if (!ws.gexec || std::memcmp(&key, &ws.gkey, sizeof(key)) != 0) {
-    if (ws.gexec) cudaGraphExecDestroy(ws.gexec);
-    ws.gexec = nullptr;
-    if (ws.graph) cudaGraphDestroy(ws.graph);
-    ws.graph = nullptr;
-    ws.gnode[0] = ws.gnode[1] = nullptr;
+  finish_args(c, g, ws, mode);
+  LaunchGraph *lg = nullptr;
+  for (LaunchGraph &x : ws.graphs)
+    if (x.exec && std::memcmp(&key, &x.key, sizeof(key)) == 0) lg = &x;
+  if (!lg) {
+    lg = &ws.graphs[0];  // the least recently used
+    for (LaunchGraph &x : ws.graphs)
+      if (x.used < lg->used) lg = &x;
+    if (lg->exec) cudaGraphExecDestroy(lg->exec);
+    lg->exec = nullptr;
+    if (lg->graph) cudaGraphDestroy(lg->graph);
+    lg->graph = nullptr;
+    lg->node[0] = lg->node[1] = nullptr;
     if (timed)
-      for (cudaEvent_t &ev : ws.gev)
+      for (cudaEvent_t &ev : lg->ev)
         if (!ev && cudaEventCreate(&ev) != cudaSuccess) return SV_ECUDA;
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SV_ECUDA;
-    const PrimeTab pt = prime_tab(c);
-    cudaError_t e = cudaMemcpyAsync(ws.reqs.p, ws.h_reqs.p, sizeof(ReqDesc) * req_copy, cudaMemcpyHostToDevice, st);
-    if (!e) e = cudaMemcpyAsync(ws.hdr.p, ws.h_hdr.p, sizeof(LaunchHeader), cudaMemcpyHostToDevice, st);
+    cudaError_t e = cudaMemcpyAsync(ws.io.p, ws.h_io.p, in_bytes, cudaMemcpyHostToDevice, st);
     // sized for the buffers (the kernel reads the launch's sizes from the header)
-    if (!e) e = launch_init(ws.hdr.p, ws.slots.p, (uint32_t)std::min<size_t>(ws.slots.cap, 1u << 20), ws.bucket_count.p,
-                            mode == 0 ? ws.stage_cnt.p : nullptr, (uint32_t)std::min<size_t>(ws.bucket_count.cap, 1u << 30),
-                            ws.reqs.p, g.mw, c->d_p, c->n_primes, p_hyb_sq(g), st);
-    if (!e && pt.n > g.i_large) {
-      BucketArgs b{};
-      b.pt = pt;
-      b.g = g;
-      b.reqs = ws.reqs.p;
-      b.hdr = ws.hdr.p;
-      b.bucket_count = ws.bucket_count.p;
-      b.bucket_data = ws.bucket_data.p;
-      e = launch_bucket_fill(b, pt.n - g.i_large, 1u << 20, 1ull << 23, fill_blocks(c), st);
-    }
-    if (!e) {
-      TileArgs t{};
-      t.pt = pt;
-      t.g = g;
-      t.reqs = ws.reqs.p;
-      t.hdr = ws.hdr.p;
-      t.slots = ws.slots.p;
-      t.list_n = ws.list_n.p;
-      t.list_k = ws.list_k.p;
-      t.fail_n = ws.fail_n.p;
-      t.strag = ws.strag.p;
-      t.strag_cap = ws.strag_cap;
-      t.bucket_count = ws.bucket_count.p;
-      t.bucket_data = ws.bucket_data.p;
-      if (mode == 0) {
-        t.stage_n = ws.stage_n.p;
-        t.stage_k = ws.stage_k.p;
-        t.stage_cnt = ws.stage_cnt.p;
-      }
-      if (timed) e = cudaEventRecordWithFlags(ws.gev[0], st, cudaEventRecordExternal);
-      if (!e) e = launch_tile_stage(c, t, mode, ws.search_all, 0xFFFFFFFFu, st);
-      if (!e && timed) e = cudaEventRecordWithFlags(ws.gev[1], st, cudaEventRecordExternal);
-    }
-    if (!e) {
-      StragArgs sa{};
-      sa.pt = pt;
-      sa.reqs = ws.reqs.p;
-      sa.hdr = ws.hdr.p;
-      sa.slots = ws.slots.p;
-      sa.list_n = ws.list_n.p;
-      sa.list_k = ws.list_k.p;
-      sa.fail_n = ws.fail_n.p;
-      sa.strag = ws.strag.p;
-      sa.strag_cap = ws.strag_cap;
-      sa.rec_t = g.rec_t;
-      if (mode == 0) {
-        sa.stage_n = ws.stage_n.p;
-        sa.stage_k = ws.stage_k.p;
-        sa.stage_cnt = ws.stage_cnt.p;
-        sa.stage_cap = g.stage_cap;
-        sa.tw = g.tw;
-        sa.tw_inv = g.tw_inv;
-      }
-      e = launch_stragglers(sa, (uint32_t)c->num_sms * 2, st);
-    }
-    if (!e && mode == 0) {
-      CompactArgs ca{};
-      ca.reqs = ws.reqs.p;
-      ca.hdr = ws.hdr.p;
-      ca.slots = ws.slots.p;
-      ca.list_n = ws.list_n.p;
-      ca.list_k = ws.list_k.p;
-      ca.stage_n = ws.stage_n.p;
-      ca.stage_k = ws.stage_k.p;
-      ca.stage_cnt = ws.stage_cnt.p;
-      ca.stage_cap = g.stage_cap;
-      e = launch_compact(ca, 4u * (uint32_t)c->num_sms, st);  // blocks of 128 tiles, grid-stride
-    }
+    if (!e && init)
+      e = launch_init(ws.hdr, ws.slots, key.n_class, nullptr, nullptr, 0, ws.reqs, g.mw, c->d_p, c->n_primes,
+                      p_hyb_sq(g), st);
+    if (!e && c->n_primes > g.i_large)
+      e = launch_bucket_fill(bucket_args(c, g, ws), c->n_primes - g.i_large, 1u << 20, 1ull << 23, fill_blocks(c), st);
+    if (!e && timed) e = cudaEventRecordWithFlags(lg->ev[0], st, cudaEventRecordExternal);
+    if (!e) e = launch_tile_stage(c, tile_args(c, g, ws, mode), mode, ws.search_all, 0xFFFFFFFFu, st);
+    if (!e && timed) e = cudaEventRecordWithFlags(lg->ev[1], st, cudaEventRecordExternal);
+    if (!e && !ws.lazy_strag) e = launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st);
+    if (!e && mode == 0) e = launch_compact(ws.compact_args, 4u * (uint32_t)c->num_sms, st);  // grid-stride
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
     if (e || e2 != cudaSuccess) {
@@ -703,34 +719,39 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
         cudaEvent_t ev = nullptr;
         if ((e4 = cudaGraphEventRecordNodeGetEvent(nodes[i], &ev))) break;
         for (int k = 0; k < 2; ++k)
-          if (ev == ws.gev[k]) ws.gnode[k] = nodes[i];
+          if (ev == lg->ev[k]) lg->node[k] = nodes[i];
       }
-      if (e4 || !ws.gnode[0] || !ws.gnode[1]) {
+      if (e4 || !lg->node[0] || !lg->node[1]) {
         cudaGraphDestroy(graph);
         return SV_ECUDA;
       }
     }
-    const cudaError_t e3 = cudaGraphInstantiate(&ws.gexec, graph, 0);
+    const cudaError_t e3 = cudaGraphInstantiate(&lg->exec, graph, 0);
     if (e3 != cudaSuccess) {
       cudaGraphDestroy(graph);
-      ws.gexec = nullptr;
+      lg->exec = nullptr;
       return SV_ECUDA;
     }
-    ws.graph = graph;  // kept: the exec's event nodes are addressed through it
-    ws.gkey = key;
+    lg->graph = graph;  // kept: the exec's event nodes are addressed through it
+    lg->key = key;
   }
+  lg->used = ++ws.graph_launches;
   if (timed) {  // fresh events for this replay's tile kernel
     cudaEvent_t a = pool_event(c), b = pool_event(c);
-    SV_TRY_CUDA(cudaGraphExecEventRecordNodeSetEvent(ws.gexec, ws.gnode[0], a));
-    SV_TRY_CUDA(cudaGraphExecEventRecordNodeSetEvent(ws.gexec, ws.gnode[1], b));
+    SV_TRY_CUDA(cudaGraphExecEventRecordNodeSetEvent(lg->exec, lg->node[0], a));
+    SV_TRY_CUDA(cudaGraphExecEventRecordNodeSetEvent(lg->exec, lg->node[1], b));
     c->kev.push_back({ws.tile_kernel_id, a, b});
   }
-  SV_TRY_CUDA(cudaGraphLaunch(ws.gexec, st));
+  if (!ws.counts_clean) {
+    SV_TRY_CUDA(cudaMemsetAsync(ws.bucket_count.p, 0, sizeof(uint32_t) * ws.bucket_count.cap, st));
+    ws.counts_clean = true;
+  }
+  SV_TRY_CUDA(cudaGraphLaunch(lg->exec, st));
   // the graph reads the staging when it runs: the next plan waits for it
   if (!ws.staged && cudaEventCreateWithFlags(&ws.staged, cudaEventDisableTiming) != cudaSuccess) return SV_ECUDA;
   SV_TRY_CUDA(cudaEventRecord(ws.staged, st));
-  c->launches += mode == 0 ? 5 : 4;
-  ws.h2d_bytes = sizeof(ReqDesc) * req_copy + sizeof(LaunchHeader);
+  c->launches += 1u + (init ? 1u : 0u) + (c->n_primes > g.i_large ? 1u : 0u) + (ws.lazy_strag ? 0u : 1u) + (mode == 0 ? 1u : 0u);
+  ws.h2d_bytes = in_bytes;
   return SV_OK;
 }
 
@@ -788,15 +809,15 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
                   cudaStream_t st, Collect *what) {
   const uint32_t n = ws.n_reqs;
   *what = kDone;
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.h_hdr.p, ws.hdr.p, sizeof(LaunchHeader), cudaMemcpyDeviceToHost, st));
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.h_slots.p, ws.slots.p, sizeof(ResultSlot) * n, cudaMemcpyDeviceToHost, st));
-  // an ordered list region is copied with the header (one wait instead of
-  // two) when it is small enough to copy whole
+  const bool short_lists = ws.io_end > ws.io_list;
+  const size_t out_bytes = short_lists ? ws.io_end - ws.io_hdr : ws.io_slots + sizeof(ResultSlot) * n - ws.io_hdr;
+  // an ordered list region of its own is copied with the header (one wait
+  // instead of two) when it is small enough to copy whole
   uint64_t spec_end = 0;
-  if (ws.ordered && outs) {
+  if (!short_lists && ws.ordered && outs) {
     for (uint32_t r = 0; r < n; ++r)
       if (outs[r] && (outs[r]->list || outs[r]->list_k))
-        spec_end = std::max<uint64_t>(spec_end, ws.h_reqs.p[r].list_off + ws.h_reqs.p[r].list_cap);
+        spec_end = std::max<uint64_t>(spec_end, ws.h_reqs[r].list_off + ws.h_reqs[r].list_cap);
     if (spec_end > kSpeculativeList) spec_end = 0;
   }
   // one range whose caller buffers are pinned host memory: its list region
@@ -804,22 +825,35 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
   // entries past the list's length are left unspecified
   bool direct = false;
   uint64_t direct_m = 0;
-  if (spec_end && n == 1 && outs[0] && is_pinned(outs[0]->list) && is_pinned(outs[0]->list_k)) {
-    direct = true;
-    direct_m = std::min<uint64_t>(ws.h_reqs.p[0].list_cap, outs[0]->list_cap);
-    const uint64_t off = ws.h_reqs.p[0].list_off;
-    if (direct_m && outs[0]->list)
-      SV_TRY_CUDA(cudaMemcpyAsync(outs[0]->list, ws.list_n.p + off, 8 * direct_m, cudaMemcpyDeviceToHost, st));
-    if (direct_m && outs[0]->list_k)
-      SV_TRY_CUDA(cudaMemcpyAsync(outs[0]->list_k, ws.list_k.p + off, direct_m, cudaMemcpyDeviceToHost, st));
-  } else if (spec_end) {
-    if (ws.h_list_n.ensure(spec_end) || ws.h_list_k.ensure(spec_end)) return SV_ENOMEM;
-    SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_n.p, ws.list_n.p, 8 * spec_end, cudaMemcpyDeviceToHost, st));
-    SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_k.p, ws.list_k.p, spec_end, cudaMemcpyDeviceToHost, st));
+  for (;;) {
+    SV_TRY_CUDA(cudaMemcpyAsync(ws.h_io.p + ws.io_hdr, ws.io.p + ws.io_hdr, out_bytes, cudaMemcpyDeviceToHost, st));
+    if (spec_end && n == 1 && outs[0] && is_pinned(outs[0]->list) && is_pinned(outs[0]->list_k)) {
+      direct = true;
+      direct_m = std::min<uint64_t>(ws.h_reqs[0].list_cap, outs[0]->list_cap);
+      const uint64_t off = ws.h_reqs[0].list_off;
+      if (direct_m && outs[0]->list)
+        SV_TRY_CUDA(cudaMemcpyAsync(outs[0]->list, ws.d_list_n + off, 8 * direct_m, cudaMemcpyDeviceToHost, st));
+      if (direct_m && outs[0]->list_k)
+        SV_TRY_CUDA(cudaMemcpyAsync(outs[0]->list_k, ws.d_list_k + off, direct_m, cudaMemcpyDeviceToHost, st));
+    } else if (spec_end) {
+      if (ws.h_list_n.ensure(spec_end) || ws.h_list_k.ensure(spec_end)) return SV_ENOMEM;
+      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_n.p, ws.d_list_n, 8 * spec_end, cudaMemcpyDeviceToHost, st));
+      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_k.p, ws.d_list_k, spec_end, cudaMemcpyDeviceToHost, st));
+    }
+    SV_TRY_CUDA(cudaStreamSynchronize(st));
+    if (!ws.lazy_strag || !ws.h_hdr->strag_count || ws.h_hdr->status) break;
+    // stragglers after all: their kernel, the lists again, and another look
+    ws.lazy_strag = false;
+    SV_TRY_CUDA(launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st));
+    c->launches++;
+    if (ws.compact_grid) {
+      SV_TRY_CUDA(launch_compact(ws.compact_args, ws.compact_grid, st));
+      c->launches++;
+    }
   }
-  SV_TRY_CUDA(cudaStreamSynchronize(st));
-  uint64_t d2h = sizeof(LaunchHeader) + sizeof(ResultSlot) * n + (direct ? 9 * direct_m : 9 * spec_end);
-  const uint32_t status = ws.h_hdr.p->status;
+  uint64_t d2h = out_bytes + (direct ? 9 * direct_m : 9 * spec_end);
+  const uint32_t status = ws.h_hdr->status;
+  if (status & (kStBadTile | kStTimeout)) ws.counts_clean = false;  // some tiles were not worked
   if (status & kStBadTile) return SV_ECUDA;
   if (status & kStTimeout) return SV_ETIMEDOUT;
   if (status & kStBucketOverflow) {
@@ -839,7 +873,7 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
   if (ws.ordered && !ws.search_all)
     for (uint32_t r = 0; r < n; ++r)
       for (int k = 1; k <= 5; ++k)
-        if (ws.h_slots.p[r].hist[k] && ws.h_slots.p[r].first_n[k] == kNoN) {
+        if (ws.h_slots[r].hist[k] && ws.h_slots[r].first_n[k] == kNoN) {
           *what = kRetryFirst;
           return SV_OK;
         }
@@ -848,7 +882,7 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
   // ordered list already holds the smallest ones and is re-run only when
   // the consumer can hold more than the device region did
   for (uint32_t r = 0; r < n; ++r) {
-    const ResultSlot &s = ws.h_slots.p[r];
+    const ResultSlot &s = ws.h_slots[r];
     if (!outs || !outs[r]) continue;
     const uint64_t limit = ws.ordered ? std::min<uint64_t>(list_want(specs[r], outs[r]), kListRetryMax) : kListRetryMax;
     if (outs[r]->list_cap && s.list_count > specs[r].list_cap && specs[r].list_cap < limit) {
@@ -860,31 +894,33 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
   uint64_t list_end = 0, fail_end = 0;
   for (uint32_t r = 0; r < n; ++r) {
     if (!outs || !outs[r]) continue;
-    const ReqDesc &d = ws.h_reqs.p[r];
-    const ResultSlot &s = ws.h_slots.p[r];
+    const ReqDesc &d = ws.h_reqs[r];
+    const ResultSlot &s = ws.h_slots[r];
     const uint64_t nl = std::min<uint64_t>(s.list_count, d.list_cap);
     const uint64_t nf = std::min<uint64_t>(s.fail_count, d.fail_cap);
     if (nl && (outs[r]->list || outs[r]->list_k)) list_end = std::max<uint64_t>(list_end, d.list_off + nl);
     if (nf && outs[r]->failures) fail_end = std::max<uint64_t>(fail_end, d.fail_off + nf);
   }
-  if (list_end <= spec_end) list_end = 0;  // already here
+  if (list_end <= spec_end || short_lists) list_end = 0;  // already here
   if (list_end || fail_end) {
     if ((list_end && (ws.h_list_n.ensure(list_end) || ws.h_list_k.ensure(list_end))) ||
         ws.h_fail_n.ensure(fail_end ? fail_end : 1))
       return SV_ENOMEM;
     if (list_end) {
-      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_n.p, ws.list_n.p, 8 * list_end, cudaMemcpyDeviceToHost, st));
-      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_k.p, ws.list_k.p, list_end, cudaMemcpyDeviceToHost, st));
+      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_n.p, ws.d_list_n, 8 * list_end, cudaMemcpyDeviceToHost, st));
+      SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_k.p, ws.d_list_k, list_end, cudaMemcpyDeviceToHost, st));
     }
     if (fail_end) SV_TRY_CUDA(cudaMemcpyAsync(ws.h_fail_n.p, ws.fail_n.p, 8 * fail_end, cudaMemcpyDeviceToHost, st));
     SV_TRY_CUDA(cudaStreamSynchronize(st));
     d2h += 9 * list_end + 8 * fail_end;
   }
+  const uint64_t *hl_n = short_lists ? (const uint64_t *)(ws.h_io.p + ws.io_list) : ws.h_list_n.p;
+  const uint8_t *hl_k = short_lists ? ws.h_io.p + ws.io_list + (ws.d_list_k - (const uint8_t *)ws.d_list_n) : ws.h_list_k.p;
   std::vector<std::pair<uint64_t, uint8_t>> v;
   for (uint32_t r = 0; r < n; ++r) {
     if (!outs || !outs[r]) continue;
     sv_range_result *o = outs[r];
-    const ResultSlot &s = ws.h_slots.p[r];
+    const ResultSlot &s = ws.h_slots[r];
     const RangeSpec &sp = specs[r];
     o->lo = sp.lo;
     o->hi = sp.hi;
@@ -902,15 +938,15 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
     o->list_len = s.list_count;
     o->fail_len = s.fail_count;
     o->list_overflow = s.list_count > o->list_cap ? 1 : 0;
-    const ReqDesc &d = ws.h_reqs.p[r];
+    const ReqDesc &d = ws.h_reqs[r];
     const uint64_t nl = std::min<uint64_t>(s.list_count, d.list_cap);
     if (nl && (o->list || o->list_k) && !direct) {
       const uint64_t m = std::min<uint64_t>(nl, o->list_cap);
       if (ws.ordered) {  // ascending already (list_compact_kernel)
-        if (o->list) std::memcpy(o->list, ws.h_list_n.p + d.list_off, 8 * m);
-        if (o->list_k) std::memcpy(o->list_k, ws.h_list_k.p + d.list_off, m);
+        if (o->list) std::memcpy(o->list, hl_n + d.list_off, 8 * m);
+        if (o->list_k) std::memcpy(o->list_k, hl_k + d.list_off, m);
       } else {
-        sort_by_n(ws.h_list_n.p + d.list_off, ws.h_list_k.p + d.list_off, nl, sp.lo, sp.hi, v);
+        sort_by_n(hl_n + d.list_off, hl_k + d.list_off, nl, sp.lo, sp.hi, v);
         for (uint64_t i = 0; i < m; ++i) {
           if (o->list) o->list[i] = v[i].first;
           if (o->list_k) o->list_k[i] = v[i].second;
@@ -988,7 +1024,7 @@ sv_status run_ranges(sv_ctx *c, std::vector<RangeSpec> &specs, sv_range_result *
     if (what == kRetryStrag) ws.strag_cap *= 4;
     if (what == kRetryList) {
       for (uint32_t r = 0; r < specs.size(); ++r) {
-        const uint64_t cnt = ws.h_slots.p[r].list_count;
+        const uint64_t cnt = ws.h_slots[r].list_count;
         if (outs && outs[r] && cnt > specs[r].list_cap) {
           uint64_t cap = std::min<uint64_t>(cnt, kListRetryMax);
           if (ws.ordered) cap = std::min<uint64_t>(cap, list_want(specs[r], outs[r]));
@@ -1085,7 +1121,7 @@ void plain_retry(sv_ctx *c, Collect what, bool sieve_retry, std::vector<RangeSpe
   if (what == kRetryStrag) c->ws.strag_cap *= 4;
   if (what == kRetryGeneral) c->ws.force_general = true;
   if (what == kRetryList) {
-    uint64_t cap = std::min<uint64_t>(c->ws.h_slots.p[0].list_count, kListRetryMax);
+    uint64_t cap = std::min<uint64_t>(c->ws.h_slots[0].list_count, kListRetryMax);
     if (c->ws.ordered) cap = std::min<uint64_t>(cap, list_want(scan[0], out));
     scan[0].list_cap = cap;
   }
@@ -1366,7 +1402,8 @@ sv_status sv_verify_range(sv_ctx *c, uint64_t lo, uint64_t hi, sv_range_result *
   std::vector<RangeSpec> specs(1);
   specs[0].lo = lo;
   specs[0].hi = hi;
-  specs[0].list_cap = out->list_cap;
+  specs[0].list_cap = list_cap_estimate(range_odd_count(lo, hi), c->cfg.record_k_threshold, out->list_cap);
+  specs[0].want_cap = out->list_cap;
   specs[0].fail_cap = std::max<uint64_t>(out->fail_cap, 64);
   const uint64_t n_odd = range_odd_count(lo, hi);
   if (out->per_n_k && n_odd) {
@@ -1399,7 +1436,8 @@ sv_status sv_verify_batch(sv_ctx *c, const uint64_t *lo, const uint64_t *hi, siz
   for (size_t i = 0; i < count; ++i) {
     specs[i].lo = lo[i];
     specs[i].hi = hi[i];
-    specs[i].list_cap = out[i].list_cap;
+    specs[i].list_cap = list_cap_estimate(range_odd_count(lo[i], hi[i]), c->cfg.record_k_threshold, out[i].list_cap);
+    specs[i].want_cap = out[i].list_cap;
     specs[i].fail_cap = std::max<uint64_t>(out[i].fail_cap, 16);
     outs[i] = &out[i];
   }

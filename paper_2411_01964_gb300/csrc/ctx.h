@@ -75,21 +75,40 @@ struct RangeSpec {
 struct GraphKey {
   const void *p[16];
   Geometry g;
-  uint32_t mode, strag_cap, search_all;
-  uint64_t req_copy;
+  uint32_t mode, strag_cap, search_all, n_class;
+  uint64_t in_bytes;
   uint32_t n_table;
   uint32_t timed;  // 1: event-record nodes bracket the tile kernel
 };
 
+// A captured launch graph and what it was captured for; a timed graph keeps
+// its event-record nodes around the tile kernel (node), whose events are
+// swapped for fresh ones before each replay.
+struct LaunchGraph {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  GraphKey key{};
+  cudaGraphNode_t node[2] = {nullptr, nullptr};
+  cudaEvent_t ev[2] = {nullptr, nullptr};  // the events recorded at capture
+  uint64_t used = 0;                       // the launch that used it last
+};
+constexpr int kGraphs = 4;  // graphs kept per workspace: launches of a few shapes alternate without capturing anew
+
 // Everything one launch needs on the device, reused across launches.
 struct Workspace {
-  DBuf<ReqDesc> reqs;
-  HBuf<ReqDesc> h_reqs;
-  DBuf<LaunchHeader> hdr;
-  HBuf<LaunchHeader> h_hdr;
-  DBuf<ResultSlot> slots;
-  HBuf<ResultSlot> h_slots;
-  DBuf<uint64_t> list_n;
+  // One block of device memory and its page-locked image hold what a launch
+  // exchanges with the host, in this order: descriptors, header, result slots
+  // and, if they are short, the lists.  One copy brings the front part in,
+  // one copy takes the back part out.
+  DBuf<unsigned char> io;
+  HBuf<unsigned char> h_io;
+  size_t io_hdr = 0, io_slots = 0, io_list = 0, io_end = 0;  // offsets; io_end == io_list: long lists, kept apart
+  ReqDesc *reqs = nullptr, *h_reqs = nullptr;
+  LaunchHeader *hdr = nullptr, *h_hdr = nullptr;
+  ResultSlot *slots = nullptr, *h_slots = nullptr;
+  uint64_t *d_list_n = nullptr;  // the lists on the device
+  uint8_t *d_list_k = nullptr;
+  DBuf<uint64_t> list_n;         // long lists
   DBuf<uint8_t> list_k;
   HBuf<uint64_t> h_list_n;
   HBuf<uint8_t> h_list_k;
@@ -120,14 +139,15 @@ struct Workspace {
   uint64_t j_max = 0;  // largest odd-multiplier count of the launch (bucket fill by j)
   uint32_t inject_bulk_timeouts = 0;  // plain-path launches still to run with their bulk loads left out (test hook)
   uint64_t h2d_bytes = 0, d2h_bytes = 0;
-  // the captured launch graph and what it was captured for; a timed graph
-  // keeps its event-record nodes around the tile kernel (gnode), whose
-  // events are swapped for fresh ones before each replay
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t gexec = nullptr;
-  GraphKey gkey{};
-  cudaGraphNode_t gnode[2] = {nullptr, nullptr};
-  cudaEvent_t gev[2] = {nullptr, nullptr};  // the events recorded at capture
+  LaunchGraph graphs[kGraphs];
+  uint64_t graph_launches = 0;
+  bool counts_clean = false;  // bucket_count is all zero (the tile kernels clear what they read)
+  // a launch without its straggler kernel, and what that kernel and the list
+  // compaction after it would have been launched with
+  bool lazy_strag = false;
+  StragArgs strag_args{};
+  CompactArgs compact_args{};
+  uint32_t compact_grid = 0;  // 0: no ordered lists
   cudaEvent_t staged = nullptr;  // recorded after the launch's reads of the pinned staging
   void release_all();
 };

@@ -567,6 +567,7 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
         sh.chunk_end = ce;
       }
       describe(s, sh, sh.desc[buf ^ 1u], D, next, gt, total, n_reqs, M);
+      a.bucket_count[gt] = 0;  // read by every thread above
     }
     // dense primes: the planned tasks of this warp; in a smaller window one
     // warp per prime, 32 consecutive strikes at a time
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
       sh.first[lane + 32] = kNone;
       if (lane < 5) sh.u[lane] = 0;
       if (lane == 0) {
-        if (ms) a.stage_cnt[gt] = ms;
+        a.stage_cnt[gt] = ms;
         if (m > ms) atomicOr(&a.hdr->status, kStListStage);
         sh.n_strag = sh.lst_cnt = 0;
       }

@@ -169,7 +169,7 @@ struct TileArgs {
   uint64_t *fail_n;
   Straggler *strag;
   uint32_t strag_cap;
-  const uint32_t *bucket_count;
+  uint32_t *bucket_count;  // read, then cleared for the next launch
   const uint32_t *bucket_data;
   // mode 0: tile t stages its list entries at [t * kStageCap, + stage_cnt[t])
   uint64_t *stage_n;

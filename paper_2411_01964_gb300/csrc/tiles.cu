@@ -197,8 +197,8 @@ __device__ __forceinline__ void strike(uint32_t *win, uint32_t b) {
 }
 
 // ---------------------------------------------------------------------------
-// init: zero the launch's counters, result slots, bucket and staged-list
-// counts; give each range of a large launch its number of table primes p
+// init: zero the launch's counters, result slots and (unless null) bucket and
+// staged-list counts; give each range of a large launch its number of table primes p
 // with p^2 < hi (Algorithm 1's "primes 3 <= p < sqrt(end)",
 // ReqDesc::n_primes) and the integer square roots of its bucket-fill interval
 // ends (ReqDesc::sq_lo, sq_hi) for the multiplier items; the host plans these
@@ -227,10 +227,11 @@ __global__ void init_kernel(LaunchHeader *hdr, ResultSlot *slots, uint32_t *buck
     R.n_primes = lo;
     R.j_max = (ph2 && R.jhi) ? (2 * R.jhi - 1) / ph2 : 0;
   }
-  for (uint32_t i = gid; i < n_tiles; i += gs) {
-    bucket_count[i] = 0;
-    if (stage_cnt) stage_cnt[i] = 0;
-  }
+  if (bucket_count)
+    for (uint32_t i = gid; i < n_tiles; i += gs) {
+      bucket_count[i] = 0;
+      if (stage_cnt) stage_cnt[i] = 0;
+    }
   for (uint32_t i = gid; i < n_slots * (uint32_t)kMaxK; i += gs) {
     slots[i / kMaxK].hist[i % kMaxK] = 0ull;
     slots[i / kMaxK].first_n[i % kMaxK] = kNoN;
@@ -1004,6 +1005,7 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
           sh.sparse_off[j] = b;
         }
       }
+      if (tid == 0) a.bucket_count[gt] = 0;  // read by every thread above; clear for the next launch
       for (uint32_t e = tid; e < nb; e += S) {
         const uint32_t b = e < S ? bv0 : (e < 2 * S ? bv1 : bd[e]);
         if (b < nbits) strike(win, b);
@@ -1098,7 +1100,7 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
           a.stage_k[(size_t)gt * kStageCap + e] = sh.lst_k[e];
         }
         if (lane == 0) {
-          if (ms) a.stage_cnt[gt] = ms;
+          a.stage_cnt[gt] = ms;
           if (m > ms) atomicOr(&a.hdr->status, kStListStage);
         }
       }
