@@ -1169,14 +1169,29 @@ sv_status collect_ranges(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_rang
   return s;
 }
 
+// The points in ws.h_points, their answers to ws.h_points_out (no wait).  Few
+// points are read from and answered into the page-locked buffers by the kernel
+// itself: two copies would take longer to start than its reads and one-byte
+// writes take (one point: 30 us a call with the copies).
+constexpr uint64_t kPointsInPlace = 2048;
+sv_status points_through_host(sv_ctx *c, uint64_t count, Workspace &ws, cudaStream_t st) {
+  const bool in_place = count <= kPointsInPlace;
+  if (!in_place) {
+    if (ws.points.ensure(count) || ws.points_out.ensure(count)) return SV_ENOMEM;
+    SV_TRY_CUDA(cudaMemcpyAsync(ws.points.p, ws.h_points.p, 8 * count, cudaMemcpyHostToDevice, st));
+  }
+  KTimer kt(c, kKPoints, st);
+  SV_TRY_CUDA(launch_points(prime_tab(c), in_place ? ws.h_points.p : ws.points.p, count,
+                            in_place ? ws.h_points_out.p : ws.points_out.p, (uint32_t)c->num_sms, st));
+  kt.done();
+  c->launches++;
+  if (!in_place) SV_TRY_CUDA(cudaMemcpyAsync(ws.h_points_out.p, ws.points_out.p, count, cudaMemcpyDeviceToHost, st));
+  return SV_OK;
+}
+
 sv_status launch_points_async(sv_ctx *c, uint64_t count, Workspace &ws, cudaStream_t st) {
   if (count == 0) return SV_OK;
-  if (ws.points.ensure(count) || ws.points_out.ensure(count)) return SV_ENOMEM;
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.points.p, ws.h_points.p, 8 * count, cudaMemcpyHostToDevice, st));
-  SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)c->num_sms, st));
-  c->launches++;
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.h_points_out.p, ws.points_out.p, count, cudaMemcpyDeviceToHost, st));
-  return SV_OK;
+  return points_through_host(c, count, ws, st);
 }
 
 sv_status run_points(sv_ctx *c, const uint64_t *points, size_t count, uint8_t *out_k, cudaStream_t st,
@@ -1184,18 +1199,10 @@ sv_status run_points(sv_ctx *c, const uint64_t *points, size_t count, uint8_t *o
   if (count == 0) return SV_OK;
   for (size_t i = 0; i < count; ++i)
     if (points[i] > c->max_hi) return SV_ERANGE;
-  if (ws.points.ensure(count) || ws.points_out.ensure(count) || ws.h_points.ensure(count) ||
-      ws.h_points_out.ensure(count))
-    return SV_ENOMEM;
+  if (ws.h_points.ensure(count) || ws.h_points_out.ensure(count)) return SV_ENOMEM;
   std::memcpy(ws.h_points.p, points, 8 * count);
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.points.p, ws.h_points.p, 8 * count, cudaMemcpyHostToDevice, st));
-  {
-    KTimer kt(c, kKPoints, st);
-    SV_TRY_CUDA(launch_points(prime_tab(c), ws.points.p, count, ws.points_out.p, (uint32_t)c->num_sms, st));
-    kt.done();
-  }
-  c->launches++;
-  SV_TRY_CUDA(cudaMemcpyAsync(ws.h_points_out.p, ws.points_out.p, count, cudaMemcpyDeviceToHost, st));
+  const sv_status s = points_through_host(c, count, ws, st);
+  if (s) return s;
   SV_TRY_CUDA(cudaStreamSynchronize(st));
   std::memcpy(out_k, ws.h_points_out.p, count);
   c->last_h2d = 8 * count;

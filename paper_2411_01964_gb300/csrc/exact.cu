@@ -151,9 +151,12 @@ __global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const u
   __shared__ uint32_t bad, n_div[K];   // bad: bit j, p^2 divides the j-th value
   __shared__ uint64_t div_inv[K][kMaxDivisors];
   __shared__ uint32_t found;
+  __shared__ uint64_t n_s;
   const uint32_t tid = threadIdx.x, T = blockDim.x;
   for (uint64_t e = blockIdx.x; e < count; e += gridDim.x) {
-    const uint64_t n = pts[e];
+    if (tid == 0) n_s = pts[e];  // (perhaps in host memory: read once)
+    __syncthreads();
+    const uint64_t n = n_s;
     uint32_t k = 0;
     if (n >= 3 && (n & 1ull)) {
       for (uint32_t k0 = 1;; k0 += K) {
