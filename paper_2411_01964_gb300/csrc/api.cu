@@ -371,7 +371,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
   uint64_t hi_max = 0;   // and the largest prime count with hi
   const uint64_t ph2 = g.p_hyb == 0xFFFFFFFFu ? 0 : (uint64_t)g.p_hyb * g.p_hyb;
   bool any_per_n = false;
-  bool all_from_bitmap = n > 0;
+  bool all_from_bitmap = n > 0, any_scan = false;
   for (uint32_t r = 0; r < n; ++r) {
     const RangeSpec &s = specs[r];
     ReqDesc d{};
@@ -421,6 +421,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
     d.bitmap_in = s.bitmap_in;
     d.bitmap_w0 = s.bitmap_w0;
     all_from_bitmap &= (s.bitmap_in != nullptr);
+    any_scan |= !s.sieve_only;
     ws.h_reqs[r] = d;
     if (n <= kHostPlanMax) {  // the result slot as the launch finds it (many ranges: by the init kernel)
       ResultSlot &slot = ws.h_slots[r];
@@ -449,7 +450,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
   ws.j_max = (ph2 && jhi_max) ? (2 * jhi_max - 1) / ph2 : 0;
   ws.any_per_n = any_per_n;
   ws.all_from_bitmap = all_from_bitmap;
-  ws.ordered = !any_per_n && g.rec_t > 5 && !ws.force_general;
+  ws.ordered = any_scan && !any_per_n && g.rec_t > 5 && !ws.force_general;  // (a sieve pass has no lists)
   return SV_OK;
 }
 
@@ -1536,7 +1537,7 @@ sv_status sv_sieve_bitmap(sv_ctx *c, uint64_t lo, uint64_t hi, uint32_t *d_bitma
   specs[0].hi = hi;
   specs[0].sieve_only = true;
   specs[0].bitmap_out = d_bitmap;
-  return run_ranges(c, specs, nullptr, c->stream, c->ws, false);
+  return run_ranges(c, specs, nullptr, c->stream, c->ws, true);
 }
 
 sv_status sv_launch_range(sv_ctx *c, uint64_t lo, uint64_t hi, uint8_t *d_per_n_k) {

@@ -196,6 +196,19 @@ __device__ __forceinline__ void strike(uint32_t *win, uint32_t b) {
   atomicAnd(&win[b >> 5], __funnelshift_l(0xFFFFFFFEu, 0xFFFFFFFEu, b));
 }
 
+// Clear bit b of the window at shared address `base`, and the same bit of
+// every step-th word after it, below nwords: three instructions per strike (a
+// mask and a bit index per strike, and shared pointers stepped in 64 bits, took
+// about ten: sv_sieve_bitmap of 2^32 integers 175 us a call, with this and one
+// graph launch instead of five kernels 149).
+__device__ __forceinline__ void strike_words(uint32_t base, uint32_t b, uint32_t step, uint32_t nwords) {
+  const uint32_t mask = __funnelshift_l(0xFFFFFFFEu, 0xFFFFFFFEu, b);
+  const uint32_t end = base + 4u * nwords;
+#pragma unroll 4
+  for (uint32_t x = base + 4u * (b >> 5); x < end; x += 4u * step)
+    asm volatile("red.shared.and.b32 [%0], %1;" ::"r"(x), "r"(mask) : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // init: zero the launch's counters, result slots and (unless null) bucket and
 // staged-list counts; give each range of a large launch its number of table primes p
@@ -758,8 +771,6 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
   const uint32_t tid = threadIdx.x, S = blockDim.x;
   const uint32_t lane = tid & 31u, warp = tid >> 5;
   const Geometry g = a.g;
-  const uint32_t total = a.hdr->total_tiles;
-  const uint32_t n_reqs = a.hdr->n_reqs;
   const uint32_t nd = g.i_dense - g.i_med;  // <= kMaxDense (host guarantees)
   // frequent exponents whose first occurrence is searched per tile: k = 1 .. kfirst
   const uint32_t kfirst = min(min(g.rec_t, g.kwin + 1u) - 1u, 5u);
@@ -776,7 +787,10 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
   bool store_pending = false;   // thread 0: a bulk store may still read the window
   build_stamp_tables<NS>(stab);
   if (PER_N) build_per_n_lut(lut);
+  const uint32_t total = a.hdr->total_tiles;
+  const uint32_t n_reqs = a.hdr->n_reqs;
   const uint32_t T = 32u * g.tw;  // a window starts T bits above the previous one
+  const uint32_t win_addr = (uint32_t)__cvta_generic_to_shared(win);
   if (tid == 0) {
     sh.n_strag = 0;
     sh.lst_cnt = 0;
@@ -951,20 +965,14 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
     // ---- 2. strikes: dense primes spread over all threads, sparse primes one
     //         thread each, large primes from the tile's bucket ---------------
     {
+      // A stride of 32 q (or a multiple) bits is whole words: a thread's
+      // strikes of one prime keep their mask, and only the word moves.
       // head primes (>= 1 strike per thread): thread tid strikes their bits
       // off + q (tid + S m)
       const uint32_t nh = min(g.n_head, nd);
       for (uint32_t d = 0; d < nh; ++d) {
         const uint32_t q = sh.dense_q[d];
-        const uint32_t step = S * q;  // <= the window's bits
-        uint32_t b = sh.dense_off[d] + tid * q;
-        // two strikes per trip, their atomics in flight together (b and step are both below the window's
-        // bits, so b + step cannot wrap)
-        for (; b + step < nbits; b += 2u * step) {
-          strike(win, b);
-          strike(win, b + step);
-        }
-        if (b < nbits) strike(win, b);
+        strike_words(win_addr, sh.dense_off[d] + tid * q, q * (S >> 5), nwords);
       }
       // the other dense primes, one warp each in a snake order over the warps
       // (their strike counts fall with p); lane l strikes off + q (l + 32 m)
@@ -973,13 +981,8 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
         for (uint32_t rd = 0;; ++rd) {
           const uint32_t d = nh + rd * nw + ((rd & 1u) ? nw - 1u - warp : warp);
           if (d >= nd) break;
-          const uint32_t q = sh.dense_q[d], step = 32u * q;  // step <= the window's bits
-          uint32_t b = sh.dense_off[d] + lane * q;
-          for (; b + step < nbits; b += 2u * step) {
-            strike(win, b);
-            strike(win, b + step);
-          }
-          if (b < nbits) strike(win, b);
+          const uint32_t q = sh.dense_q[d];
+          strike_words(win_addr, sh.dense_off[d] + lane * q, q, nwords);
         }
       }
       // a full window's strikes carry to the next window: its first struck
