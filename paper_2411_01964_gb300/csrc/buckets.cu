@@ -11,8 +11,12 @@
 //     struck bit, then the thread walks the further hits (for a launch of
 //     few ranges, the blocks of the smallest primes, which have the most
 //     hits, are cut into segments of the range, one item each);
-//   * multiplier items (slice, request): primes p >= p_hyb, reached through
-//     their odd multipliers j (j p^2 in the range) and the prime bitmap.
+//   * multiplier items (slice, request or chunk of requests): primes p >=
+//     p_hyb, reached through their odd multipliers j (j p^2 in the range) and
+//     the prime bitmap.
+// Both are bound by the arithmetic that finds out that there is no hit, which
+// is the answer for nearly every (prime or multiplier, range) of a batch; a
+// quick test comes first in either.
 // A bucket slot is reserved with a global atomic that returns the slot; a
 // Barrett thread reserves the slots of up to four hits together, so that
 // their round trips overlap instead of queueing one behind the other.
@@ -39,8 +43,13 @@ constexpr uint32_t kMaxSeg = 64;  // a power of two
 constexpr uint32_t kMaxSplitBlocks = 16;  // prime blocks that may be cut
 constexpr uint32_t kMaxSplitExtra = kMaxSplitBlocks * (kMaxSeg - 1);
 
-struct FillReq {
-  uint64_t A, E;  // struck bits wanted: [A, E)
+// A range (or a segment of one) as the Barrett items see it.  A, len and
+// top_hi are what the quick test reads (one 16-byte load).
+struct __align__(16) FillReq {
+  uint64_t A;       // struck bits wanted: [A, E)
+  uint32_t len;     // E - A, at most 2^32 - 1
+  uint32_t top_hi;  // floor(E / 2^32) + 1
+  uint64_t E;
   int64_t w0;
   uint32_t tile_base, n_tiles, n_primes, pad;
 };
@@ -151,6 +160,8 @@ __device__ void fill_barrett_item(const BucketArgs &a, FillReq *s_req, uint32_t 
       f.A = a0 < f.E ? a0 : f.E;
       if (f.E - f.A > len) f.E = f.A + len;
     }
+    f.len = f.E > f.A ? (uint32_t)min(f.E - f.A, (uint64_t)0xFFFFFFFFu) : 0u;
+    f.top_hi = (uint32_t)(f.E >> 32) + 1u;
     f.w0 = R.w0;
     f.tile_base = R.tile_base;
     f.n_tiles = R.n_tiles;
@@ -163,21 +174,23 @@ __device__ void fill_barrett_item(const BucketArgs &a, FillReq *s_req, uint32_t 
   if (pi >= prime_end) return;
   const uint64_t p = a.pt.p[pi];
   const uint64_t q = p * p, mu = a.pt.mu[pi];
-  // two ranges per step: their first-strike reductions are independent
-  // chains of 64-bit multiplies, so they overlap; a hit (rare for most
-  // primes and ranges) is then walked range by range
-  // (only the bounds are held across the pair; a walk reads the rest of its
-  // range from shared memory)
-  uint32_t r = 0;
-  for (; r + 1 < nr; r += 2) {
-    const uint64_t A0 = s_req[r].A, A1 = s_req[r + 1].A;
-    const uint64_t J0 = A0 + first_strike(A0, q, mu), J1 = A1 + first_strike(A1, q, mu);
-    if (J0 < s_req[r].E && pi < s_req[r].n_primes && s_req[r].n_tiles) barrett_walk(a, s_req[r], J0, q);
-    if (J1 < s_req[r + 1].E && pi < s_req[r + 1].n_primes && s_req[r + 1].n_tiles)
-      barrett_walk(a, s_req[r + 1], J1, q);
-  }
-  if (r < nr) {
-    const uint64_t J = s_req[r].A + first_strike(s_req[r].A, q, mu);
+  // Most primes have no hit in most ranges, so a quick test comes before the
+  // first-strike reduction.  With c = (q - 1)/2 the struck bits are J = c (mod
+  // q).  Let o be the distance from A to the first one, A + o = c + k q.  As q mu
+  // = 2^64 - 1 - rho with 0 <= rho < q, modulo 2^64
+  //   g := (c - A) mu = o mu + k (1 + rho),   0 <= k (1 + rho) <= A + o,
+  // so a hit, o < len, has g <= len mu + E, of which the high words are
+  // compared (rounded up, and no smaller when the right side passes 2^64).  A
+  // range without a hit passes with a chance of about len/q + E/2^64.  Ten
+  // instructions; the reduction takes about thirty-five.
+  const uint64_t cmu = ((q - 1) >> 1) * mu;
+  const uint32_t mu_hi1 = (uint32_t)(mu >> 32) + 1u;
+#pragma unroll 4
+  for (uint32_t r = 0; r < nr; ++r) {
+    const uint4 f = *reinterpret_cast<const uint4 *>(&s_req[r]);  // A, len, top_hi
+    const uint64_t A = (uint64_t)f.y << 32 | f.x;
+    if ((uint64_t)(uint32_t)((cmu - A * mu) >> 32) > (uint64_t)f.z * mu_hi1 + f.w) continue;
+    const uint64_t J = A + first_strike(A, q, mu);
     if (J < s_req[r].E && pi < s_req[r].n_primes && s_req[r].n_tiles) barrett_walk(a, s_req[r], J, q);
   }
 }
@@ -259,14 +272,14 @@ __device__ __forceinline__ uint32_t interval_word(const BucketArgs &a, uint64_t 
   return mm;
 }
 
-// Slice s of nsl of range r's odd multipliers j (j p^2 in the range, p >= p_hyb).
+// Slice s of nsl of range r's small odd multipliers j < 2 kWarpJ (j p^2 in the
+// range, p >= p_hyb).
 // The smallest multipliers have the longest p intervals (and the most hits).
 // A long range (>= 2^30 odd numbers) spreads the bitmap words of all its
 // small multipliers over the threads of all slices, one word each (the
 // intervals and their word counts are computed once per item);
 // a shorter one gives each small j to one warp, lanes striding over words.
-// Larger j take one thread each.
-__device__ void fill_mult_item(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_t s, uint32_t nsl, uint32_t r) {
+__device__ void fill_small_mult(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_t s, uint32_t nsl, uint32_t r) {
   const Geometry &g = a.g;
   const ReqDesc &R = a.reqs[r];
   if (R.n_tiles == 0 || R.n_primes <= g.i_hyb) return;  // uniform over the block
@@ -276,11 +289,8 @@ __device__ void fill_mult_item(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_
   const uint64_t ph = g.p_hyb;
   const uint64_t mlo = 2 * A + 1, mhi = 2 * E - 1;
   const uint64_t jmax = R.j_max;  // floor(mhi / p_hyb^2), planned once per range
-  // a slice past the range's multipliers has nothing to do (a long range
-  // spreads its small multipliers' words over every slice, below)
-  if (E - A < (1ull << 30) && (uint64_t)s * (blockDim.x >> 5) >= kWarpJ &&
-      2 * (kWarpJ + (uint64_t)s * blockDim.x) + 1 > jmax)
-    return;  // uniform over the block
+  // (a long range spreads its small multipliers' words over every slice, below)
+  if (E - A < (1ull << 30) && (uint64_t)s * (blockDim.x >> 5) >= kWarpJ) return;  // uniform over the block
   const uint64_t p_top = a.pt.p[R.n_primes - 1];  // primes with p^2 < hi
   const uint64_t w_end = a.pt.bits_words;
   if (E - A >= (1ull << 30)) {
@@ -330,24 +340,75 @@ __device__ void fill_mult_item(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_
       for (uint64_t w = (b0 >> 5) + lane; w <= w_last; w += 32) emit_word(a, R, interval_word(a, w, b0, b1), w, j);
     }
   }
-  for (uint64_t t = kWarpJ + (uint64_t)s * blockDim.x + threadIdx.x; 2 * t + 1 <= jmax;
-       t += (uint64_t)nsl * blockDim.x) {
+}
+
+// Slice s of nsl of the larger odd multipliers j = 2t + 1, t >= kWarpJ, of the
+// nr ranges from r0 on: one thread per multiplier, which keeps the reciprocal
+// square root of j for all the ranges.  For most (j, range) no p lies in the
+// interval at all: the largest p with j p^2 <= mhi (estimated from the range's
+// root, corrected in steps of j (2p + 1)) has j p^2 < mlo.  That takes about
+// 20 instructions; only otherwise are both ends computed and the bitmap read.
+constexpr uint32_t kMultReqChunk = 16;
+struct MultReq {
+  uint64_t mlo, mhi, jmax;
+  uint32_t sq_hi, pad;
+};
+__device__ void fill_large_mult(const BucketArgs &a, MultReq *s_mult, uint32_t s, uint32_t nsl, uint32_t r0, uint32_t nr) {
+  const Geometry &g = a.g;
+  __syncthreads();  // s_mult holds the previous item's ranges
+  if (threadIdx.x < nr) {
+    const ReqDesc &R = a.reqs[r0 + threadIdx.x];
+    const int64_t ws = R.w0 - (int64_t)g.mw;
+    const uint64_t A = 32ull * (uint64_t)(ws < 0 ? 0 : ws), E = R.jhi;
+    MultReq m;
+    m.mlo = 2 * A + 1;
+    m.mhi = E > A ? 2 * E - 1 : 0;
+    m.jmax = R.n_tiles && R.n_primes > g.i_hyb && E > A ? R.j_max : 0;
+    m.sq_hi = R.sq_hi;
+    m.pad = 0;
+    s_mult[threadIdx.x] = m;
+  }
+  __syncthreads();
+  uint64_t jm = 0;
+  for (uint32_t r = 0; r < nr; ++r) jm = max(jm, s_mult[r].jmax);
+  for (uint64_t t = kWarpJ + (uint64_t)s * blockDim.x + threadIdx.x; 2 * t + 1 <= jm; t += (uint64_t)nsl * blockDim.x) {
     const uint64_t j = 2 * t + 1;
-    uint64_t b0, b1;
-    if (!p_interval(mlo, mhi, R.sq_lo, R.sq_hi, j, ph, p_top, &b0, &b1)) continue;
-    const uint64_t w_last = min(b1 >> 5, w_end - 1);
-    for (uint64_t wd = b0 >> 5; wd <= w_last; wd += 4) {  // four words in flight
-      uint32_t m[4];
+    const uint64_t z = rsqrt_fix(j);
+    const uint32_t z_hi = (uint32_t)(z >> 32);
+    for (uint32_t r = 0; r < nr; ++r) {
+      const MultReq m = s_mult[r];
+      if (j > m.jmax) continue;
+      // floor(sqrt(mhi / j)): sq_hi z / 2^63 is a few units below it at most
+      uint64_t p = ((uint64_t)m.sq_hi * z_hi) >> 31;
+      uint64_t v = j * p * p, step = j * (2 * p + 1);
+      while (v + step <= m.mhi) {
+        v += step;
+        step += 2 * j;
+      }
+      while (v > m.mhi) {  // (the estimate does not exceed the root; kept for safety)
+        step -= 2 * j;
+        v -= step;
+      }
+      if (v < m.mlo) continue;
+      const ReqDesc &R = a.reqs[r0 + r];
+      const uint64_t p_top = a.pt.p[R.n_primes - 1];  // primes with p^2 < hi
+      uint64_t b0, b1;
+      if (!p_interval(m.mlo, m.mhi, R.sq_lo, R.sq_hi, j, g.p_hyb, p_top, &b0, &b1)) continue;
+      const uint64_t w_last = min(b1 >> 5, a.pt.bits_words - 1);
+      for (uint64_t wd = b0 >> 5; wd <= w_last; wd += 4) {  // four words in flight
+        uint32_t mm[4];
 #pragma unroll
-      for (uint32_t u = 0; u < 4; ++u) m[u] = wd + u <= w_last ? interval_word(a, wd + u, b0, b1) : 0u;
+        for (uint32_t u = 0; u < 4; ++u) mm[u] = wd + u <= w_last ? interval_word(a, wd + u, b0, b1) : 0u;
 #pragma unroll
-      for (uint32_t u = 0; u < 4; ++u) emit_word(a, R, m[u], wd + u, j);
+        for (uint32_t u = 0; u < 4; ++u) emit_word(a, R, mm[u], wd + u, j);
+      }
     }
   }
 }
 
-// The item space: jx slices x jy requests of multiplier items, then px prime
-// blocks x py request chunks of Barrett items (host-chosen upper bounds).
+// The item space: jx slices x jy requests of small multipliers, jx slices x
+// chunks of requests of larger ones, then px prime blocks x py request chunks
+// of Barrett items (host-chosen upper bounds).
 // Each is trimmed to what the launch's header asks for, so that a captured
 // launch sized for its buffers wastes no block on absent work.
 struct FillItems {
@@ -356,6 +417,7 @@ struct FillItems {
 
 __global__ void __launch_bounds__(kFillThreads, kFillBlocksPerSm) bucket_fill_kernel(BucketArgs a, FillItems fi) {
   __shared__ FillReq s_req[kFillReqChunk];
+  __shared__ MultReq s_mult[kMultReqChunk];
   __shared__ uint64_t s_iv[kWarpJ + 1][3];  // small multipliers: interval bits, first word's rank; [kWarpJ][2]: total
   const Geometry &g = a.g;
   const uint32_t n_reqs = a.hdr->n_reqs;
@@ -397,14 +459,24 @@ __global__ void __launch_bounds__(kFillThreads, kFillBlocksPerSm) bucket_fill_ke
   const uint32_t jx_need = (uint32_t)min((jm / 2 + kFillThreads) / kFillThreads, (uint64_t)fi.jx);
   const uint32_t jx = (max_primes > g.i_hyb && g.p_hyb != 0xFFFFFFFFu) ? min(fi.jx, max(jx_need, 8u)) : 0u;
   const uint32_t jy = min(fi.jy, n_reqs);
-  const uint32_t n_mult = jx * jy;  // <= 64 * 1024
+  // small multipliers: a warp each, unless a long range spreads their words
+  const uint32_t jxs = a.hdr->fill_span >= (1ull << 30) ? jx : min(jx, (uint32_t)kWarpJ / (kFillThreads / 32));
+  const uint32_t n_small = jxs * jy;  // <= 64 * 1024
+  // larger ones: a chunk of ranges per item, so that a multiplier's reciprocal
+  // square root is computed once for them, while there are items enough for
+  // every block (up to 32 ranges: one range each)
+  const uint32_t cr = min(max(n_reqs / 32u, 1u), kMultReqChunk), n_cr = (n_reqs + cr - 1u) / cr;
+  const uint32_t n_mult = n_small + min(jx * n_cr, 0x40000000u);
   // Blocks take items round robin.  The multiplier items come first, slice
   // by slice: the low slices hold the small multipliers, the costliest
   // items, and consecutive items land on different blocks.
   for (uint32_t it = blockIdx.x; it < n_mult + n_bar; it += gridDim.x) {
-    if (it < n_mult) {
+    if (it < n_small) {
       // item (s, ry) covers slice s of the ranges ry + jy k
-      for (uint32_t r = it % jy; r < n_reqs; r += jy) fill_mult_item(a, s_iv, it / jy, jx, r);
+      for (uint32_t r = it % jy; r < n_reqs; r += jy) fill_small_mult(a, s_iv, it / jy, jxs, r);
+    } else if (it < n_mult) {
+      const uint32_t m = it - n_small, r0 = m % n_cr * cr;
+      fill_large_mult(a, s_mult, m / n_cr, jx, r0, min(cr, n_reqs - r0));
     } else {
       const uint32_t m = it - n_mult;
       // item (x, rcy) covers (prime block, segment) items x + px i and
