@@ -286,6 +286,7 @@ cudaError_t launch_tile_stage(const sv_ctx *c, const TileArgs &t, int mode, bool
   s.magic = stream_magic(kStreamRun * g.threads);
   s.sparse_room = g.i_large - g.i_dense;
   s.search_all = search_all ? 1u : 0u;
+  s.one = 1;
   plan_strikes(c->h_p.data() + g.i_med, g.i_dense - g.i_med, s.sparse_room, g.threads, &s.plan);
   return launch_stream_tiles(s, grid, st);
 }

@@ -143,7 +143,7 @@ __device__ __forceinline__ uint32_t seg_count(const BucketArgs &a, uint32_t pb, 
 
 // Primes of prime block pb (one per thread) against segment seg of nseg of
 // each range of request chunk rc.
-__device__ void fill_barrett_item(const BucketArgs &a, FillReq *s_req, uint32_t pb, uint32_t seg, uint32_t nseg,
+__device__ __noinline__ void fill_barrett_item(const BucketArgs &a, FillReq *s_req, uint32_t pb, uint32_t seg, uint32_t nseg,
                                   uint32_t rc, uint32_t n_reqs, uint32_t prime_end) {
   const uint32_t r0 = rc * kFillReqChunk;
   const uint32_t nr = min(kFillReqChunk, n_reqs - r0);
@@ -279,7 +279,7 @@ __device__ __forceinline__ uint32_t interval_word(const BucketArgs &a, uint64_t 
 // small multipliers over the threads of all slices, one word each (the
 // intervals and their word counts are computed once per item);
 // a shorter one gives each small j to one warp, lanes striding over words.
-__device__ void fill_small_mult(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_t s, uint32_t nsl, uint32_t r) {
+__device__ __noinline__ void fill_small_mult(const BucketArgs &a, uint64_t (*s_iv)[3], uint32_t s, uint32_t nsl, uint32_t r) {
   const Geometry &g = a.g;
   const ReqDesc &R = a.reqs[r];
   if (R.n_tiles == 0 || R.n_primes <= g.i_hyb) return;  // uniform over the block
@@ -353,7 +353,7 @@ struct MultReq {
   uint64_t mlo, mhi, jmax;
   uint32_t sq_hi, pad;
 };
-__device__ void fill_large_mult(const BucketArgs &a, MultReq *s_mult, uint32_t s, uint32_t nsl, uint32_t r0, uint32_t nr) {
+__device__ __noinline__ void fill_large_mult(const BucketArgs &a, MultReq *s_mult, uint32_t s, uint32_t nsl, uint32_t r0, uint32_t nr) {
   const Geometry &g = a.g;
   __syncthreads();  // s_mult holds the previous item's ranges
   if (threadIdx.x < nr) {

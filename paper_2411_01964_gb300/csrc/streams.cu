@@ -24,12 +24,15 @@
 // look-back up to k = kwin and leave the rest to the exact test; 4. add the
 // tile's counts to its range's slot and stage its listed n, as tiles.cu does.
 //
-// Bound: integer issue (25 thousand warp instructions per tile of 585504 odd n,
-// 0.60 issued per scheduler and cycle, logic pipe 51% busy) and the barriers
-// between the phases.  [2^40, 2^40 + 2^34): 492 us, against 601 us of
-// tile_kernel<0, 4> in the linear layout; of the 492 the search takes about
-// 260, the dense strikes 65, the stamp 60, the rest is per-tile set-up and
-// sparse primes.  Blocks of 512 threads, two per SM: four of 256 take 518.
+// Bound: integer issue and the logic pipe (22 thousand warp instructions per
+// tile of 585504 odd n, 0.65 issued per scheduler and cycle, the logic pipe half
+// busy, over 70% in the search), then the barriers between the phases.
+// [2^40, 2^40 + 2^34): 398 us, against 601 us of tile_kernel<0, 4> in the linear
+// layout.  Blocks of 512 threads, two per SM: four of 256 took 4% longer, a tile
+// queue in chunks of 6 or 12 tiles instead of 8 1% and 5%.  Counting the n left
+// after k = 4 by their bits' columns, with a recount where two met, instead of
+// word by word: 9% longer (they come in clusters).  Larger dense primes one per
+// warp instead of eight: 2%.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -132,7 +135,7 @@ __device__ __forceinline__ void lds4(uint32_t addr, uint32_t *v) {
 __device__ __forceinline__ void sts(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-// Three-input logic, one instruction each: a ^ b ^ c, the majority, a | b | c, (a & b) | c.
+// Three-input logic, one instruction each: a ^ b ^ c, the majority, (a & b) | c.
 __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
@@ -141,11 +144,6 @@ __device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
 __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("lop3.b32 %0, %1, %2, %3, 0xE8;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-__device__ __forceinline__ uint32_t or3(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xFE;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
 __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
@@ -197,17 +195,25 @@ __device__ __noinline__ void finish_word(const Win win, uint32_t i, uint32_t u, 
   }
 }
 
-// Sums of population counts by carry-save addition: each pair of words costs
-// two three-input logic operations and one count instead of two counts (a
-// count issues at an eighth of the logic rate).
+// Sums of population counts.  The logic pipe bounds the search, the count
+// pipe (an eighth of its rate) comes next, the multiply-add pipe is nearly
+// idle: the sums are multiply-adds by a 1 that the compiler cannot see, and
+// carry-save addition, one logic operation per word, halves the counts where
+// that evens the two pipes out (k = 1, 2 and 3; the sets of k = 4 are counted word
+// by word).
+__device__ __forceinline__ uint32_t add_count(uint32_t x, uint32_t one, uint32_t sum) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(__popc(x)), "r"(one), "r"(sum));
+  return d;
+}
 struct Counter {
   uint32_t ones = 0, twos = 0;  // ones: one bit per column still to be counted; twos: counted pairs
-  __device__ __forceinline__ void add(const uint32_t (&u)[4]) {
+  __device__ __forceinline__ void add(const uint32_t (&u)[4], uint32_t one) {
     const uint32_t a = maj3(ones, u[0], u[1]);
     ones = xor3(ones, u[0], u[1]);
     const uint32_t b = maj3(ones, u[2], u[3]);
     ones = xor3(ones, u[2], u[3]);
-    twos += __popc(a) + __popc(b);
+    twos = add_count(b, one, add_count(a, one, twos));
   }
   __device__ __forceinline__ uint32_t total() const { return 2u * twos + __popc(ones); }
 };
@@ -217,26 +223,18 @@ __device__ __forceinline__ uint32_t left_after_4(const Win win, uint32_t i, uint
   return vm & win.look(i, 1) & win.look(i, 2) & win.look(i, 4) & win.look(i, 8);
 }
 
-// How many n of a run are left after k = 4, when scan_run's sum of them met
-// two in one column.
-__device__ __noinline__ uint32_t count_u4(const Win win, uint32_t i0, uint32_t vm) {
-  uint32_t c = 0;
-  for (uint32_t i = i0; i < i0 + kRun; ++i) c += __popc(left_after_4(win, i, vm));
-  return c;
-}
-
 // The search over one thread's run of words i0 .. i0 + kRun - 1, for the n of
 // the bits vm.  With z the struck words, the n left after k = 1, 2, 3, 4, 5
 // are z[i-1], & z[i-2], & z[i-4], & z[i-8], & z[i-16]: one logic operation per
 // word and k.  The sets of k = 1..4 are counted (hist[k] = U_(k-1) - U_k).
 // When a lane has an n left after k = 5 among kPiece words (one piece in
-// 380), it queues the piece.  FIRST5: the tile may hold the range's first n
-// of k = 5.
+// 380), it queues the piece.  MASK false: vm is all ones.  FIRST5: the tile
+// may hold the range's first n of k = 5.
 constexpr uint32_t kPiece = 12;
 static_assert(kRun % kPiece == 0 && kPiece % 4 == 0, "a run is whole pieces");
-template <bool FIRST5>
+template <bool MASK, bool FIRST5>
 __device__ __forceinline__ void scan_run(const Win win, uint32_t base, uint32_t i0, uint32_t vm, StreamShared &sh,
-                                         uint32_t warp, uint32_t (&U)[4]) {
+                                         uint32_t warp, uint32_t one, uint32_t (&U)[4]) {
   uint32_t z[kRun + 16];
   const uint32_t at = base + 4u * i0;
   {
@@ -249,7 +247,7 @@ __device__ __forceinline__ void scan_run(const Win win, uint32_t base, uint32_t 
     for (uint32_t j = 0; j < 16; ++j) z[j] <<= up;
   }
   Counter c1, c2, c3;
-  uint32_t ones4 = 0, over4 = 0;  // rarely more than one bit per column: checked, not carried
+  uint32_t n4 = 0;
 #pragma unroll
   for (uint32_t h = 0; h < kRun; h += kPiece) {
     uint32_t left = 0;
@@ -260,7 +258,7 @@ __device__ __forceinline__ void scan_run(const Win win, uint32_t base, uint32_t 
 #pragma unroll
       for (uint32_t j = 0; j < 4; ++j) {
         const uint32_t *p = z + 16 + g + j;
-        u1[j] = p[-1] & vm;
+        u1[j] = MASK ? p[-1] & vm : p[-1];
         u2[j] = u1[j] & p[-2];
         u3[j] = u2[j] & p[-4];
         u4[j] = u3[j] & p[-8];
@@ -270,14 +268,11 @@ __device__ __forceinline__ void scan_run(const Win win, uint32_t base, uint32_t 
           if (f) atomicMin(&sh.first[5], (uint32_t)(__ffs(f) - 1) * win.M + i0 + g + j);
         }
       }
-      c1.add(u1);
-      c2.add(u2);
-      c3.add(u3);
-      const uint32_t a = maj3(ones4, u4[0], u4[1]);
-      ones4 = or3(ones4, u4[0], u4[1]);
-      const uint32_t b = maj3(ones4, u4[2], u4[3]);
-      ones4 = or3(ones4, u4[2], u4[3]);
-      over4 = or3(over4, a, b);
+      c1.add(u1, one);
+      c2.add(u2, one);
+      c3.add(u3, one);
+#pragma unroll
+      for (uint32_t j = 0; j < 4; ++j) n4 = add_count(u4[j], one, n4);
     }
     if (__any_sync(0xFFFFFFFFu, left)) {
       if (left) {
@@ -289,21 +284,25 @@ __device__ __forceinline__ void scan_run(const Win win, uint32_t base, uint32_t 
   U[0] = c1.total();
   U[1] = c2.total();
   U[2] = c3.total();
-  U[3] = __popc(ones4);
-  if (__any_sync(0xFFFFFFFFu, over4)) {
-    if (over4) U[3] = count_u4(win, i0, vm);
-  }
+  U[3] = n4;
 }
 
-// One warp's piece of one dense prime: lane l strikes the window bits
-// r + q (l + 32 m), m = m0 .. m0 + n - 1.  q is odd and M a multiple of 32, so
-// the lanes' words lie on 32 banks.  A step of 32 q moves a lane dw words up
-// and db streams on (one more when it runs past word M); past the last stream
-// its mask is shifted out and it strikes nothing.
+// One warp's piece of a dense prime, or of kGroup consecutive ones with kLanes
+// lanes each (the larger primes, whose strikes would leave most lanes of a
+// warp idle or each pay a warp's set-up): lane l of a prime's L lanes strikes
+// the window bits r + q (l + L m), m = m0 .. m0 + n - 1.  q is odd and M a
+// multiple of 32, so one prime's lanes lie on different banks.  A step of L q
+// moves a lane dw words up and db streams on (one more when it runs past word
+// M); past the last stream its mask is shifted out and it strikes nothing.
+constexpr uint32_t kGroup = 8, kLanes = 32 / kGroup;
+__device__ __forceinline__ bool grouped(uint32_t q, uint32_t M) { return 32u * M < 128u * q; }  // under 128 strikes
 __device__ __forceinline__ void strike_task(const Win win, uint32_t base, const StreamShared &sh, const StrikeTask t,
-                                            uint32_t lane) {
-  const uint4 c = sh.dense[t.d];  // q, dw in bytes, db
-  const uint32_t bit = sh.dense_r[t.d] + c.x * (lane + 32u * t.m0);
+                                            uint32_t lane, uint32_t nd) {
+  const bool group = t.d & kStrikeGroup;
+  const uint32_t d = group ? min((t.d & ~kStrikeGroup) + lane / kLanes, nd - 1u) : t.d;
+  const uint32_t l = group ? lane % kLanes : lane + 32u * t.m0;
+  const uint4 c = sh.dense[d];  // q, dw in bytes, db
+  const uint32_t bit = sh.dense_r[d] + c.x * l;
   const uint32_t M4 = 4u * win.M;
   uint32_t x = 0, mask = 0;
   if (bit < 32u * win.M) {
@@ -315,8 +314,8 @@ __device__ __forceinline__ void strike_task(const Win win, uint32_t base, const 
   x += base;
   const uint32_t end = base + M4;
   strike_at(x, mask);
-  if (c.z == 0) {  // q < M / 32
-#pragma unroll 4
+  if (!group && c.z == 0) {  // q < M / 32
+#pragma unroll 8
     for (uint32_t n = t.n - 1u; n; --n)
       asm volatile(
           "{\n.reg .pred p;\n"
@@ -349,8 +348,7 @@ __device__ __forceinline__ void strike_task(const Win win, uint32_t base, const 
 // next; the last 4 tiles per CTA go one at a time, which evens out the CTAs'
 // finishing times (the split of tiles.cu, where it was measured).
 __device__ __forceinline__ void chunk_range(uint32_t j, uint32_t total, uint32_t ctas, uint32_t *s, uint32_t *e) {
-  const uint32_t chunk = total >= 128u * ctas ? 12u : 6u;
-  const uint32_t reserve = 4u * ctas;
+  const uint32_t chunk = 8u, reserve = 4u * ctas;
   const uint32_t n_big = total > reserve ? (total - reserve) / chunk : 0u;
   uint64_t b, f;
   if (j < n_big) {
@@ -504,7 +502,8 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
   }
   for (uint32_t d = tid; d < nd; d += S) {
     const uint32_t p = a.pt.p[g.i_med + d], q = p * p;  // q <= 32 M / kDenseMinHits
-    sh.dense[d] = make_uint4(q, 4u * ((32u * q) % M), (32u * q) / M, T % q);
+    const uint32_t L = grouped(q, M) ? kLanes : 32u;
+    sh.dense[d] = make_uint4(q, 4u * ((L * q) % M), (L * q) / M, T % q);
   }
   if (tid < nwarps) sh.q_cnt[tid] = 0;
   if (tid == 0) {
@@ -573,7 +572,7 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
     // warp per prime, 32 consecutive strikes at a time
     if (full) {
       for (uint32_t x = s.plan.start[warp]; x < s.plan.start[warp + 1]; ++x)
-        strike_task(win, win_addr, sh, s.plan.task[x], lane);
+        strike_task(win, win_addr, sh, s.plan.task[x], lane, nd);
     } else {
       for (uint32_t d = warp; d < nd; d += nwarps) {
         const uint32_t q = sh.dense[d].x;
@@ -615,8 +614,9 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
       const uint32_t i0 = kRun * tid;
       const uint32_t vm = bits_from(i0 >= il ? bl : bl + 1u) & ~bits_from(i0 + kRun <= ih ? bh + 1u : bh);
       uint32_t U[4];
-      if (search) scan_run<true>(win, win_addr, i0, vm, sh, warp, U);
-      else scan_run<false>(win, win_addr, i0, vm, sh, warp, U);
+      if (search) scan_run<true, true>(win, win_addr, i0, vm, sh, warp, s.one, U);
+      else if (__all_sync(0xFFFFFFFFu, vm == 0xFFFFFFFFu)) scan_run<false, false>(win, win_addr, i0, vm, sh, warp, s.one, U);
+      else scan_run<true, false>(win, win_addr, i0, vm, sh, warp, s.one, U);
 #pragma unroll
       for (uint32_t k = 0; k < 4; ++k) {
         const uint32_t x = __reduce_add_sync(0xFFFFFFFFu, U[k]);
@@ -769,7 +769,7 @@ void plan_strikes(const uint32_t *primes, uint32_t nd, uint32_t n_sparse, uint32
   };
   std::memset(plan, 0, sizeof(*plan));
   const uint32_t M = kRun * threads, nw = threads / 32;
-  constexpr uint32_t kSetup = 24, kStep = 6, kSparseSetup = 30, kSparseStrike = 16, kDescribe = 250;
+  constexpr uint32_t kSetup = 24, kStep = 6, kSparseSetup = 30, kSparseStrike = 30, kDescribe = 250;
   uint32_t load[kMaxStrikeWarps] = {0};
   load[0] = kDescribe;
   uint32_t sum = kDescribe;
@@ -779,17 +779,24 @@ void plan_strikes(const uint32_t *primes, uint32_t nd, uint32_t n_sparse, uint32
     load[nw - 1 - (j0 / 32) % nw] += c;
     sum += c;
   }
-  // steps of 32 strikes r + q (l + 32 m) below 32 M, r < q
-  auto steps_of = [&](uint32_t d) { return (M - 1) / (primes[d] * primes[d]) + 1; };
-  for (uint32_t d = 0; d < nd; ++d) sum += kSetup + kStep * steps_of(d);
+  // steps of L strikes r + q (l + L m) below 32 M, r < q
+  auto steps_of = [&](uint32_t d, uint32_t L) { return (32 * M - 1) / (L * primes[d] * primes[d]) + 1; };
+  uint32_t n_single = 0;  // the first primes have a warp each (see grouped())
+  while (n_single < nd && 32ull * M >= 128ull * primes[n_single] * primes[n_single]) ++n_single;
+  for (uint32_t d = 0; d < n_single; ++d) sum += kSetup + kStep * steps_of(d, 32);
+  for (uint32_t d = n_single; d < nd; d += kGroup) sum += kSetup + kStep * steps_of(d, kLanes);
   const uint32_t share = std::max(sum / nw, 1u);
   Job jobs[kMaxStrikeTasks];
   uint32_t nj = 0;
-  for (uint32_t d = 0; d < nd; ++d) {
-    const uint32_t steps = steps_of(d);
+  for (uint32_t d = n_single; d < nd; d += kGroup) {  // (the last group's spare lanes repeat prime nd - 1: harmless)
+    const uint32_t steps = steps_of(d, kLanes);
+    jobs[nj++] = {kSetup + kStep * steps, {0, (uint8_t)(d | kStrikeGroup), (uint8_t)steps}};
+  }
+  for (uint32_t d = 0; d < n_single; ++d) {
+    const uint32_t steps = steps_of(d, 32);
     // as many pieces as the task table can still hold
     uint32_t pieces = std::max(1u, (2 * kStep * steps + share - 1) / share);
-    pieces = std::min(std::min(pieces, steps), kMaxStrikeTasks - nj - (nd - 1 - d));
+    pieces = std::min(std::min(pieces, steps), kMaxStrikeTasks - nj - (n_single - 1 - d));
     for (uint32_t h = 0; h < pieces; ++h) {
       const uint32_t m0 = steps * h / pieces, m1 = steps * (h + 1) / pieces;
       jobs[nj++] = {kSetup + kStep * (m1 - m0), {(uint16_t)m0, (uint8_t)d, (uint8_t)(m1 - m0)}};

@@ -246,8 +246,9 @@ constexpr uint32_t kStreamStampStride = 2704;  // words per stamp table (one tab
 constexpr uint32_t kStreamMarginWords = 9;  // the margin is a multiple of 9 words = 288 bits, so that it ends
                                             // between two threads' runs
 // A warp's piece of one dense prime's strikes: steps m0 .. m0 + n - 1 of 32
-// strikes each.
+// strikes each; or (d with kStrikeGroup) n steps of a group of primes from d on.
 constexpr uint32_t kMaxStrikeTasks = 160, kMaxStrikeWarps = 16;
+constexpr uint8_t kStrikeGroup = 0x80;
 struct StrikeTask {
   uint16_t m0;
   uint8_t d, n;
@@ -261,6 +262,7 @@ struct StreamArgs {
   const uint32_t *stamp;   // kStreamSizes stamp tables
   uint32_t magic;          // stream_magic of the window's words
   uint32_t sparse_room;    // sparse primes the block has room for (>= i_large - i_dense)
+  uint32_t one;            // 1 (see add_count)
   uint32_t search_all;     // 1: every tile searches the first occurrences of k <= 5, not only a range's first
   StrikePlan plan;
 };
