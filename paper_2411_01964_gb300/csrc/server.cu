@@ -57,6 +57,7 @@ struct Request {
 
 struct Item {
   uint64_t ticket, lo, hi;
+  sv_range_result *whole;  // the chunk is its whole request, whose result this is (null: one of several chunks)
 };
 struct PItem {
   uint64_t ticket, first, count, off;
@@ -178,6 +179,7 @@ class Server {
     if (empty) {
       r.issued_all = true;
       complete(r);
+      cv_done_.notify_all();
     } else {
       queue_.push_back(t);
     }
@@ -329,7 +331,8 @@ class Server {
           sp.list_cap = lc;
           sp.want_cap = r.r.result->list_cap;
           sp.fail_cap = 64;
-          s.items.push_back({r.ticket, clo, chi});
+          const bool whole = clo == r.r.lo && chi == r.r.hi;
+          s.items.push_back({r.ticket, clo, chi, whole ? r.r.result : nullptr});
           s.specs.push_back(sp);
           odd += n;
           tiles += t;
@@ -371,9 +374,12 @@ class Server {
 
   // Enqueues slot s's launch (mu_ not held).
   sv_status start(Slot &s) {
+    // the points first: behind the ranges they would wait for room until the
+    // next slot's tile kernel, which fills the GPU meanwhile, is done, and this
+    // slot's results with them
     sv_status st = SV_OK;
-    if (!s.items.empty()) st = launch_ranges_async(c_, s.specs, s.ws, s.st);
-    if (!st && s.npoints) st = launch_points_async(c_, s.npoints, s.ws, s.st);
+    if (s.npoints) st = launch_points_async(c_, s.npoints, s.ws, s.st);
+    if (!st && !s.items.empty()) st = launch_ranges_async(c_, s.specs, s.ws, s.st);
     if (cudaEventRecord(s.ev, s.st) != cudaSuccess && !st) st = SV_ECUDA;
     return st;
   }
@@ -388,6 +394,10 @@ class Server {
     s.fbuf.resize(n);
     std::vector<sv_range_result *> ptrs(n);
     for (size_t i = 0; i < n; ++i) {
+      if (s.items[i].whole) {  // straight into the caller's buffers (valid until the ticket is polled)
+        ptrs[i] = s.items[i].whole;
+        continue;
+      }
       s.lbuf[i].resize(std::max<uint64_t>(s.specs[i].list_cap, 1));
       s.kbuf[i].resize(std::max<uint64_t>(s.specs[i].list_cap, 1));
       s.fbuf[i].resize(64);
@@ -405,6 +415,7 @@ class Server {
       if (!st && retry) {
         // an overflow: give the chunks full room and repeat them, blocking
         for (size_t i = 0; i < n; ++i) {
+          if (s.items[i].whole) continue;  // the caller's own buffers
           const uint64_t full = s.outs[i].list_len > s.specs[i].list_cap ? s.outs[i].list_len : 0;
           if (full) {
             s.specs[i].list_cap = full;
@@ -427,6 +438,11 @@ class Server {
       if (it == reqs_.end()) continue;
       Request &r = it->second;
       if (st) r.status = st;
+      if (s.items[i].whole) {
+        if (!st && !r.status) odd_done_ += s.items[i].whole->n_odd;
+        if (--r.outstanding == 0 && r.issued_all) finished(r);
+        continue;
+      }
       const sv_range_result &o = s.outs[i];
       if (!st) {
         for (int k = 0; k < kMaxK; ++k) {
@@ -454,6 +470,15 @@ class Server {
     s.items.clear();
     s.pitems.clear();
     s.npoints = 0;
+    cv_done_.notify_all();  // once for all of the launch's requests
+  }
+
+  // The request's result is written: it may be polled (mu_ held; the caller
+  // notifies).
+  void finished(Request &r) {
+    r.state = Request::kDone;
+    ++completed_;
+    lat_us_.push_back(std::chrono::duration<double, std::micro>(Clock::now() - r.t_submit).count());
   }
 
   // Writes the merged result into the caller's buffers (mu_ held).
@@ -493,10 +518,7 @@ class Server {
     r.list.clear();
     r.list.shrink_to_fit();
     r.fails.clear();
-    r.state = Request::kDone;
-    ++completed_;
-    lat_us_.push_back(std::chrono::duration<double, std::micro>(Clock::now() - r.t_submit).count());
-    cv_done_.notify_all();
+    finished(r);
   }
 
   void loop() {
