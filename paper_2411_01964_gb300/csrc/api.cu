@@ -302,6 +302,7 @@ PrimeTab prime_tab(const sv_ctx *c) {
   pt.mu = c->d_mu;
   pt.inv = c->d_inv;
   pt.lim = c->d_lim;
+  pt.word = c->d_word;
   pt.bits = c->d_pbits;
   pt.bits_words = c->pbits_words;
   pt.n = c->n_primes;
@@ -1331,6 +1332,7 @@ void sv_destroy(sv_ctx *c) {
   cudaFree(c->d_inv);
   cudaFree(c->d_lim);
   cudaFree(c->d_pbits);
+  cudaFree(c->d_word);
   cudaFree(c->d_stamp);
   for (auto &k : c->kev) {
     cudaEventDestroy(k.a);
@@ -1361,13 +1363,23 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
   cudaError_t e = build_prime_table(pmax, &d_p, &d_mu, &d_inv, &d_lim, &d_bits, &bits_words, &n, &n_div, c->stream);
   if (e == cudaErrorMemoryAllocation) return SV_ENOMEM;
   if (e != cudaSuccess) return SV_ECUDA;
+  PrimeWord *d_word = nullptr;
   auto free_table = [&] {
+    cudaFree(d_word);
     cudaFree(d_p);
     cudaFree(d_mu);
     cudaFree(d_inv);
     cudaFree(d_lim);
     cudaFree(d_bits);
   };
+  if (cudaMalloc((void **)&d_word, sizeof(PrimeWord) * (size_t)prime_words(n_div)) != cudaSuccess) {
+    free_table();
+    return SV_ENOMEM;
+  }
+  if (launch_prime_words(d_p, d_inv, n_div, d_word, c->stream) != cudaSuccess) {
+    free_table();
+    return SV_ECUDA;
+  }
   if (!c->d_stamp) {  // the stream layout's stamp tables (they depend on nothing)
     uint32_t *d_stamp = nullptr;
     if (cudaMalloc((void **)&d_stamp, 4ull * kStreamStampStride * kStreamSizes) != cudaSuccess) {
@@ -1392,6 +1404,8 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
   cudaFree(c->d_inv);
   cudaFree(c->d_lim);
   cudaFree(c->d_pbits);
+  cudaFree(c->d_word);
+  c->d_word = d_word;
   c->d_p = d_p;
   c->d_mu = d_mu;
   c->d_inv = d_inv;
@@ -1413,7 +1427,7 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
     c->inv_sq_suffix[j] = c->inv_sq_suffix[j + 1] + 1.0 / ((double)c->h_p[j] * (double)c->h_p[j]);
   c->pmax = pmax;
   c->max_hi = max_hi;
-  c->launches += 5;
+  c->launches += 6;
   return SV_OK;
 }
 

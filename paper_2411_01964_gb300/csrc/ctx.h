@@ -193,6 +193,7 @@ struct sv_ctx {
   uint64_t *d_mu = nullptr, *d_inv = nullptr, *d_lim = nullptr;
   uint32_t *d_pbits = nullptr;  // odd-prime bitmap of the table's range
   uint64_t pbits_words = 0;
+  sv::PrimeWord *d_word = nullptr;  // the 32-bit divisibility test's constants
   uint32_t *d_stamp = nullptr;  // the stream layout's stamp tables (streams.cu)
   uint32_t n_primes = 0, n_div = 0;
   std::vector<uint32_t> h_p;

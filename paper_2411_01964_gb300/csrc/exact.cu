@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "strike.h"
 #include "sv_internal.h"
@@ -118,34 +119,79 @@ cudaError_t launch_stragglers(const StragArgs &a, uint32_t grid, cudaStream_t st
 }
 
 // ---- point queries -------------------------------------------------------------
-// Both kernels test a prime with the high word of t = s p^-1 mod 2^64 alone:
-// p | s means t <= lim, hence t_hi <= lim_hi; the rare candidates (and the
-// rarer false ones, t_hi = lim_hi) are decided with both words.  That is
-// three multiplies and a compare per prime and value.  Primes somewhat past
-// the cube root of s may be tested too: dividing one out leaves r = 1, a
-// prime, or (r = p^2) finds p^2 | s, so the test stays exact.
-__device__ __forceinline__ bool maybe_divides(uint64_t s, uint64_t inv, uint32_t lim_hi) {
+// Both kernels rule a prime p out with 32-bit arithmetic.  With s = s1 2^32 + s0
+// and r = 2^32 mod p, v = s1 r + s0 is s modulo p; if p divides it, v = p k with
+// k <= s1 + (2^32 - 1)/p < 2^32, so that k is the low word of v times the low
+// word of p^-1:
+//   p | s  =>  (s1 r + s0) p^-1 mod 2^32 <= s1 + floor(2^32 / p) + 1,
+// two multiplies, an addition and a compare.  Other primes pass with a chance
+// of about 1/p + s1/2^32; who passes is decided by the whole 64-bit test.  From
+// 2^52 on, where s1 lets too many pass, the high word of t = s p^-1 mod 2^64 is
+// compared instead (p | s means t <= lim, hence t_hi <= lim_hi).
+// Primes somewhat past the cube root of s may be tested too: dividing one out
+// leaves r = 1, a prime, or (r = p^2) finds p^2 | s, so the test stays exact.
+// The 32-bit test's constants lie side by side, one 16-byte load per prime
+// (PrimeTab::word): its multiplies, at a quarter of the logic rate, are to be
+// what bounds the kernels, not addresses and loads.
+constexpr uint64_t kShortTest = 1ull << 52;
+__device__ __forceinline__ bool maybe_divides_short(uint64_t s, const PrimeWord &w) {
+  const uint32_t s0 = (uint32_t)s, s1 = (uint32_t)(s >> 32);
+  return (s1 * w.r + s0) * w.inv <= s1 + (w.lim + 1u);
+}
+__device__ __forceinline__ bool maybe_divides_long(uint64_t s, uint64_t inv, uint32_t lim_hi) {
   const uint32_t s0 = (uint32_t)s, s1 = (uint32_t)(s >> 32), i0 = (uint32_t)inv, i1 = (uint32_t)(inv >> 32);
   return __umulhi(s0, i0) + s0 * i1 + s1 * i0 <= lim_hi;
 }
-
-__device__ __forceinline__ uint32_t lim_high(const PrimeTab &pt, uint32_t i) {
-  return reinterpret_cast<const uint32_t *>(pt.lim)[2u * i + 1u];  // little endian
+// Which of the K values may be divisible by prime i (below the padded table's end).
+template <bool SHORT, int K>
+__device__ __forceinline__ bool any_may_divide(const PrimeTab &pt, uint32_t i, const PrimeWord &w, const uint64_t (&s)[K]) {
+  bool any = false;
+  if (SHORT) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) any |= maybe_divides_short(s[j], w);
+  } else {
+    const uint64_t inv = i < pt.n_div ? pt.inv[i] : 1ull;
+#pragma unroll
+    for (int j = 0; j < K; ++j) any |= maybe_divides_long(s[j], inv, w.lim);
+  }
+  return any;
 }
 
+// The table of the 32-bit test, padded by words that divide next to nothing (p
+// = 2^32 - 1 lies above every cube root).
+__global__ void prime_words_kernel(const uint32_t *p, const uint64_t *inv, uint32_t n_div, uint32_t n_out, PrimeWord *out) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_out) return;
+  PrimeWord w{0u, 1u, 0u, 0xFFFFFFFFu};
+  if (i < n_div) {
+    const uint32_t q = (uint32_t)((1ull << 32) / p[i]);
+    w = PrimeWord{0u - p[i] * q, (uint32_t)inv[i], q, p[i]};
+  }
+  out[i] = w;
+}
+cudaError_t launch_prime_words(const uint32_t *p, const uint64_t *inv, uint32_t n_div, PrimeWord *out, cudaStream_t st) {
+  const uint32_t n = prime_words(n_div);
+  prime_words_kernel<<<(n + 255) / 256, 256, 0, st>>>(p, inv, n_div, n, out);
+  return cudaGetLastError();
+}
+
+// p^3 <= x for a word's prime (p < 2^21: no overflow; the padding's is above)
+__device__ __forceinline__ bool cube_le(uint32_t p, uint64_t x) { return p < (1u << 21) && (uint64_t)p * p * p <= x; }
+
 // r = s less its prime divisors up to the cube root: squarefree unless r is a
-// square above 1
+// square above 1 (an odd square is 1 modulo 8)
 __device__ __forceinline__ bool cofactor_squarefree(uint64_t r) {
-  if (r == 1) return true;
+  if (r == 1 || (r & 7u) != 1) return true;
   const uint64_t x = isqrt_u64(r);
   return x * x != r;
 }
 
 constexpr uint32_t kMaxDivisors = 16;  // a product of 16 odd primes exceeds 2^62
 
-// Few points: a block per point, its threads striding the primes, and K
-// exponents at a time, so that one pass over the primes mostly suffices.
-template <int K>
+// A block per point, its threads striding the primes (U per thread and step,
+// their loads in flight together), and K exponents at a time: with few points,
+// so that one pass over the primes mostly suffices.
+template <int K, int U>
 __global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const uint64_t *pts, uint64_t count,
                                                             uint8_t *out) {
   __shared__ uint32_t bad, n_div[K];   // bad: bit j, p^2 divides the j-th value
@@ -174,28 +220,31 @@ __global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const u
           const uint32_t kj = k0 + (uint32_t)j;
           s[j] = kj < 63 && (1ull << kj) < n ? n - (1ull << kj) : 1ull;  // (1: never the answer, see below)
         }
-        for (uint32_t base = 0; base < pt.n_div; base += T) {
-          const uint64_t pb = pt.p[base];
-          if (pb * pb * pb > n) break;  // primes ascend (p < 2^21: no overflow)
-          const uint32_t i = base + tid;
-          if (i >= pt.n_div) continue;
-          const uint64_t inv = pt.inv[i];
-          const uint32_t lh = lim_high(pt, i);
-          bool any = false;
+        auto walk = [&](auto short_test) {
+          constexpr bool kShort = decltype(short_test)::value;
+          for (uint32_t base = tid; base < pt.n_div; base += U * T) {  // (the table is padded by a step)
+            PrimeWord w[U];
 #pragma unroll
-          for (int j = 0; j < K; ++j) any |= maybe_divides(s[j], inv, lh);
-          if (any) {
-            const uint64_t lim = pt.lim[i];
+            for (int u = 0; u < U; ++u) w[u] = pt.word[base + (uint32_t)u * T];
+            if (!cube_le(w[0].p, n)) break;  // primes ascend
 #pragma unroll
-            for (int j = 0; j < K; ++j) {
-              const uint64_t t = s[j] * inv;
-              if (t > lim) continue;
-              if (t * inv <= lim) atomicOr(&bad, 1u << j);
-              const uint32_t d = atomicAdd(&n_div[j], 1u);
-              if (d < kMaxDivisors) div_inv[j][d] = inv;
+            for (int u = 0; u < U; ++u) {
+              const uint32_t i = base + (uint32_t)u * T;
+              if (!any_may_divide<kShort>(pt, i, w[u], s) || i >= pt.n_div) continue;
+              const uint64_t lim = pt.lim[i], inv = pt.inv[i];
+#pragma unroll
+              for (int j = 0; j < K; ++j) {
+                const uint64_t t = s[j] * inv;
+                if (t > lim) continue;
+                if (t * inv <= lim) atomicOr(&bad, 1u << j);
+                const uint32_t d = atomicAdd(&n_div[j], 1u);
+                if (d < kMaxDivisors) div_inv[j][d] = inv;
+              }
             }
           }
-        }
+        };
+        if (n < kShortTest) walk(std::true_type());
+        else walk(std::false_type());
         __syncthreads();
         if (tid < 32) {  // lane j decides the j-th value
           bool ok = false;
@@ -285,43 +334,46 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
 #pragma unroll
     for (int j = 0; j < kSlots; ++j) top = s[j] > top ? s[j] : top;
     uint32_t bad = 0;
-    for (uint32_t base = 32; base < pt.n_div; base += 64) {
-      const uint64_t pb = pt.p[base];
-      if (pb * pb * pb > top) break;
-      uint64_t inv[2];
-      uint32_t lh[2];
-      bool any = false;
+    // the primes to walk: those with p^3 <= top
+    uint32_t n_walk = 0;
+    for (uint32_t hi = pt.n_div; n_walk < hi;) {
+      const uint32_t mid = (n_walk + hi) >> 1;
+      if (cube_le(pt.word[mid].p, top)) n_walk = mid + 1u;
+      else hi = mid;
+    }
+    auto walk = [&](auto short_test) {
+      constexpr bool kShort = decltype(short_test)::value;
+      for (uint32_t i0 = 32u + lane; i0 < n_walk + lane; i0 += 64) {  // (the table is padded by a step)
+        PrimeWord w[2];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const uint32_t i = base + 32u * u + lane;
-        inv[u] = i < pt.n_div ? pt.inv[i] : 0ull;  // (0 divides nothing: t = 0 is ruled out below)
-        lh[u] = i < pt.n_div ? lim_high(pt, i) : 0u;
-      }
+        for (int u = 0; u < 2; ++u) w[u] = pt.word[i0 + 32u * u];
+        bool any = false;
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int j = 0; j < kSlots; ++j) any |= maybe_divides(s[j], inv[u], lh[u]);
-      if (__any_sync(0xFFFFFFFFu, any)) {
+        for (int u = 0; u < 2; ++u) any |= any_may_divide<kShort>(pt, i0 + 32u * u, w[u], s);
+        if (!__any_sync(0xFFFFFFFFu, any)) continue;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const uint32_t i = base + 32u * u + lane;
-          const uint64_t lim = i < pt.n_div ? pt.lim[i] : 0ull;
+          const uint32_t i = i0 + 32u * u;
+          if (!__any_sync(0xFFFFFFFFu, any_may_divide<kShort>(pt, i, w[u], s))) continue;
+          const uint64_t inv = i < pt.n_div ? pt.inv[i] : 0ull, lim = i < pt.n_div ? pt.lim[i] : 0ull;
 #pragma unroll
           for (int j = 0; j < kSlots; ++j) {
-            const uint64_t t = s[j] * inv[u];
+            const uint64_t t = s[j] * inv;
             const bool div = i < pt.n_div && t <= lim;
             uint32_t m = __ballot_sync(0xFFFFFFFFu, div);
             if (!m) continue;
-            if (__any_sync(0xFFFFFFFFu, div && t * inv[u] <= lim)) bad |= 1u << j;
+            if (__any_sync(0xFFFFFFFFu, div && t * inv <= lim)) bad |= 1u << j;
             while (m) {
               const int src = __ffs(m) - 1;
               m &= m - 1;
-              r[j] *= __shfl_sync(0xFFFFFFFFu, inv[u], src);
+              r[j] *= __shfl_sync(0xFFFFFFFFu, inv, src);
             }
           }
         }
       }
-    }
+    };
+    if (top < kShortTest) walk(std::true_type());
+    else walk(std::false_type());
 #pragma unroll
     for (int j = 0; j < kSlots; ++j) {
       if (e[j] == ~0ull) continue;
@@ -336,22 +388,23 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
 }
 
 // Bound: few points by the latency of one pass over the primes (about 10^4 for
-// n near 2^50, ten per thread of a block), many by the multiplies (three per
-// prime and value).  One warp per point, with two 64-bit products, 64-bit
-// compares and two votes per 32 primes, took 143 us a call for one point (now
-// 30), 170 for 1024 (48) and 962 for 65536 on the device (372; with the whole
-// 64-bit product instead of its high word 396).
-// The lines: a block of 1024 threads per point while two fit every SM; smaller
-// blocks while a wave or two of them covers the points; then, with a thousand
-// points per SM's warps, the loads shared by four points.
+// n near 2^50, ten per thread of a block), many by the multiplies (two per
+// prime and value, a quarter of the logic rate).  One warp per point, with two
+// 64-bit products, 64-bit compares and two votes per 32 primes, took 962 us on
+// the device for 65536 points; the high word of the 64-bit product alone 372;
+// the 32-bit test 213.  1024 points: 21 us before the 32-bit test, 19 now.
+// The lines, with both sides measured: a block of 1024 threads per point while
+// two fit every SM (304 points: 11 us; blocks of 256 with two exponents 15);
+// those (7218 points: 66 us, four points per warp 66; 2048: 26 and 52) up to 48
+// points per SM; then a warp per four points (16384 points: 70 us, blocks 138).
 cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t num_sms,
                           cudaStream_t st) {
   if (count == 0) return cudaSuccess;
   const uint64_t sms = num_sms;
   if (count <= 2 * sms)
-    points_block_kernel<4><<<(uint32_t)count, 1024, 0, st>>>(pt, pts, count, out);
-  else if (count <= 24 * sms)
-    points_block_kernel<2><<<(uint32_t)count, 256, 0, st>>>(pt, pts, count, out);
+    points_block_kernel<4, 2><<<(uint32_t)count, 1024, 0, st>>>(pt, pts, count, out);
+  else if (count <= 48 * sms)
+    points_block_kernel<2, 4><<<(uint32_t)count, 256, 0, st>>>(pt, pts, count, out);
   else
     points_warp_kernel<<<(uint32_t)std::min<uint64_t>((count + 8 * kSlots - 1) / (8 * kSlots), 4 * sms), 256, 0, st>>>(
         pt, pts, count, out);

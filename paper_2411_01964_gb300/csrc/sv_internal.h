@@ -34,6 +34,14 @@ enum : uint32_t {
 // tile kernel's shared buffer and the stride of the per-tile staging slots.
 constexpr uint32_t kStageCap = 128;
 
+// The constants of the 32-bit divisibility test (exact.cu) of one prime: 2^32
+// mod p, p^-1 mod 2^32, floor(2^32 / p), p.
+struct __attribute__((aligned(16))) PrimeWord {
+  uint32_t r, inv, lim, p;
+};
+// Words of the padded table: a walk's step reads at most 2048 past the end.
+constexpr uint32_t prime_words(uint32_t n_div) { return n_div + 2048u; }
+
 // Resident table of the odd primes 3 <= p <= pmax (ascending), structure of
 // arrays.  mu[i] = floor((2^64-1) / p^2) is the Barrett (1986) constant for
 // x mod p^2; inv[i] = p^-1 mod 2^64 and lim[i] = floor((2^64-1)/p) give the
@@ -45,6 +53,7 @@ struct PrimeTab {
   const uint64_t *mu;
   const uint64_t *inv;
   const uint64_t *lim;
+  const PrimeWord *word;  // the first n_div primes' constants of the 32-bit test, padded (prime_words)
   const uint32_t *bits;  // bit i of the bitmap <-> odd 2i+1 is prime (up to the table's limit)
   uint64_t bits_words;
   uint32_t n;
@@ -274,6 +283,7 @@ size_t stream_static_smem();
 cudaError_t stream_kernel_setup(int optin);
 cudaError_t launch_stream_tiles(const StreamArgs &s, uint32_t grid, cudaStream_t st);
 cudaError_t launch_stragglers(const StragArgs &a, uint32_t grid, cudaStream_t st);
+cudaError_t launch_prime_words(const uint32_t *p, const uint64_t *inv, uint32_t n_div, PrimeWord *out, cudaStream_t st);
 cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t num_sms,
                           cudaStream_t st);
 uint64_t host_isqrt(uint64_t x);  // floor(sqrt(x)), exact (host)

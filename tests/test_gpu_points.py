@@ -20,17 +20,26 @@ def mixed_points(count):
     return (pts[-count:] if count < len(pts) // 2 else pts * (count // len(pts) + 1))[:count]
 
 
-@pytest.mark.parametrize("count", [1, 2, 33, 304, 305, 3648, 3649, 3680, 12345])
+@pytest.mark.parametrize("count", [1, 2, 33, 304, 305, 3648, 7296, 7297, 7400, 12345])
 def test_point_counts(gpu, orc, count):
     pts = mixed_points(count)
     assert len(pts) == count
     assert np.array_equal(gpu.min_k(pts), orc.min_k(pts))
 
 
+@pytest.mark.parametrize("count", [40, 400, 8000])
+def test_points_around_the_32_bit_test(orc, count):
+    # below 2^52 primes are ruled out in 32 bits, from there on in 64
+    pts = [(1 << 52) + d for d in range(-39, 41, 2)] + inputs.random_points(6, count, 1 << 51, 1 << 53)
+    pts = pts[:count]
+    with Verifier(max_hi=(1 << 53) + 1) as v:
+        assert np.array_equal(v.min_k(pts), orc.min_k(pts))
+
+
 def test_small_tables(orc):
     # tables with fewer primes than one step takes
     for max_hi in (30, 4000, 1 << 20):
         with Verifier(max_hi=max_hi) as v:
-            for count in (5, 400, 4000):
+            for count in (5, 400, 8000):
                 pts = [i % max_hi for i in range(count)]
                 assert np.array_equal(v.min_k(pts), orc.min_k(pts))
