@@ -610,7 +610,30 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
     uint32_t il, bl, ih, bh;
     win.split(vlo, &il, &bl);
     win.split(vhi, &ih, &bh);  // vhi = nbits: stream 32, word 0
-    if (kRun * 32u * warp < win.M) {
+    if (!full) {
+      // a small window: its words one by one, so that every warp has some (a
+      // range of 23457 integers 45 to 42 us a call; one warp's runs would be
+      // the latency of the tile)
+      uint32_t U[5] = {0, 0, 0, 0, 0};
+      for (uint32_t i = tid; i < win.M; i += S) {
+        uint32_t u = bits_from(i >= il ? bl : bl + 1u) & ~bits_from(i < ih ? bh + 1u : bh);
+        if (!u) continue;
+#pragma unroll
+        for (uint32_t k = 1; k <= 5; ++k) {
+          const uint32_t z = win.look(i, 1u << (k - 1));
+          if (k == 5 && search && (u & ~z)) atomicMin(&sh.first[5], (uint32_t)(__ffs(u & ~z) - 1) * win.M + i);
+          u &= z;
+          U[k - 1] += __popc(u);
+        }
+        if (u) finish_word(win, i, u, 6, a, sh, D.wbit, D.req_idx);
+      }
+      __syncwarp();
+#pragma unroll
+      for (uint32_t k = 0; k < 5; ++k) {
+        const uint32_t x = __reduce_add_sync(0xFFFFFFFFu, U[k]);
+        if (lane == 0 && x) atomicAdd(&sh.u[k], x);
+      }
+    } else {
       const uint32_t i0 = kRun * tid;
       const uint32_t vm = bits_from(i0 >= il ? bl : bl + 1u) & ~bits_from(i0 + kRun <= ih ? bh + 1u : bh);
       uint32_t U[4];
@@ -645,7 +668,7 @@ __global__ void __launch_bounds__(512, 2) stream_kernel(const __grid_constant__ 
         }
       }
     }
-    if (il % kRun || ih % kRun) {  // (not inside a range: the margin is a multiple of kRun)
+    if (full && (il % kRun || ih % kRun)) {  // (not inside a range: the margin is a multiple of kRun)
       const uint32_t run_l = il / kRun, run_h = ih / kRun;
       // [e0, e1): the start of the range inside its run; [f0, f1): its end
       uint32_t e0 = vlo, e1 = vlo, f0 = vhi, f1 = vhi;
