@@ -374,7 +374,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
   uint64_t span_max = 0;  // the longest range, in bits
   uint64_t hi_max = 0;   // and the largest prime count with hi
   const uint64_t ph2 = g.p_hyb == 0xFFFFFFFFu ? 0 : (uint64_t)g.p_hyb * g.p_hyb;
-  bool any_per_n = false;
+  bool any_per_n = false, all_per_n = n > 0;
   bool all_from_bitmap = n > 0, any_scan = false;
   for (uint32_t r = 0; r < n; ++r) {
     const RangeSpec &s = specs[r];
@@ -414,6 +414,7 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
     if (nt && d.jhi - d.jlo > span_max) span_max = d.jhi - d.jlo;
     d.per_n_k = s.d_per_n;
     any_per_n |= (s.d_per_n != nullptr);
+    all_per_n &= (s.d_per_n != nullptr);
     d.list_off = list_total;
     d.list_cap = s.list_cap;
     list_total += s.list_cap;
@@ -454,7 +455,8 @@ sv_status plan(sv_ctx *c, const std::vector<RangeSpec> &specs, const Geometry &g
   ws.j_max = (ph2 && jhi_max) ? (2 * jhi_max - 1) / ph2 : 0;
   ws.any_per_n = any_per_n;
   ws.all_from_bitmap = all_from_bitmap;
-  ws.ordered = any_scan && !any_per_n && g.rec_t > 5 && !ws.force_general;  // (a sieve pass has no lists)
+  // (a sieve pass has no lists)
+  ws.ordered = any_scan && any_per_n == all_per_n && g.rec_t > 5 && !ws.force_general;
   return SV_OK;
 }
 
@@ -469,19 +471,19 @@ bool ensure_stage(Workspace &ws) {
 }
 
 // The device buffers of the planned launch.
-sv_status ensure_buffers(Workspace &ws, const Geometry &g, int mode) {
+sv_status ensure_buffers(Workspace &ws, const Geometry &g) {
   const size_t tiles = ws.total_tiles ? ws.total_tiles : 1;
   const size_t counts = ws.bucket_count.cap;
   if (ws.fail_n.ensure(ws.fail_total ? ws.fail_total : 1) || ws.strag.ensure(ws.strag_cap) ||
       ws.bucket_count.ensure(tiles) || ws.bucket_data.ensure(tiles * g.bucket_cap))
     return SV_ENOMEM;
   if (ws.bucket_count.cap != counts) ws.counts_clean = false;  // grown (perhaps in place)
-  if (mode == 0 && !ensure_stage(ws)) return SV_ENOMEM;
+  if (ws.ordered && !ensure_stage(ws)) return SV_ENOMEM;
   return SV_OK;
 }
 
 // What the straggler and compaction kernels of the planned launch take.
-void finish_args(const sv_ctx *c, const Geometry &g, Workspace &ws, int mode) {
+void finish_args(const sv_ctx *c, const Geometry &g, Workspace &ws) {
   StragArgs &s = ws.strag_args;
   s = StragArgs{};
   s.pt = prime_tab(c);
@@ -495,7 +497,7 @@ void finish_args(const sv_ctx *c, const Geometry &g, Workspace &ws, int mode) {
   s.strag_cap = ws.strag_cap;
   s.rec_t = g.rec_t;
   ws.compact_grid = 0;
-  if (mode != 0) return;
+  if (!ws.ordered) return;
   s.stage_n = ws.stage_n.p;
   s.stage_k = ws.stage_k.p;
   s.stage_cnt = ws.stage_cnt.p;
@@ -517,7 +519,7 @@ void finish_args(const sv_ctx *c, const Geometry &g, Workspace &ws, int mode) {
 }
 
 // The arguments of the fill and tile kernels of the planned launch.
-TileArgs tile_args(const sv_ctx *c, const Geometry &g, const Workspace &ws, int mode) {
+TileArgs tile_args(const sv_ctx *c, const Geometry &g, const Workspace &ws) {
   TileArgs t{};
   t.pt = prime_tab(c);
   t.g = g;
@@ -531,7 +533,7 @@ TileArgs tile_args(const sv_ctx *c, const Geometry &g, const Workspace &ws, int 
   t.strag_cap = ws.strag_cap;
   t.bucket_count = ws.bucket_count.p;
   t.bucket_data = ws.bucket_data.p;
-  if (mode == 0) {
+  if (ws.ordered) {
     t.stage_n = ws.stage_n.p;
     t.stage_k = ws.stage_k.p;
     t.stage_cnt = ws.stage_cnt.p;
@@ -592,7 +594,7 @@ struct KTimer {
 sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) {
   const uint32_t n = ws.n_reqs;
   const int mode = launch_mode(ws);
-  const sv_status bs = ensure_buffers(ws, g, mode);
+  const sv_status bs = ensure_buffers(ws, g);
   if (bs) return bs;
   ws.bucket_cap = g.bucket_cap;
   const size_t in_bytes = ws.io_slots;  // descriptors and header (the init kernel sets the slots)
@@ -602,7 +604,7 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
   SV_TRY_CUDA(cudaEventRecord(ws.staged, st));
   {
     KTimer kt(c, kKInit, st);
-    SV_TRY_CUDA(launch_init(ws.hdr, ws.slots, n, ws.bucket_count.p, mode == 0 ? ws.stage_cnt.p : nullptr,
+    SV_TRY_CUDA(launch_init(ws.hdr, ws.slots, n, ws.bucket_count.p, ws.ordered ? ws.stage_cnt.p : nullptr,
                             ws.total_tiles, ws.reqs, g.mw, c->d_p, c->n_primes, p_hyb_sq(g), st));
     kt.done();
   }
@@ -618,11 +620,11 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
   if (ws.total_tiles) {
     {
       KTimer kt(c, ws.tile_kernel_id, st);
-      SV_TRY_CUDA(launch_tile_stage(c, tile_args(c, g, ws, mode), mode, ws.search_all, ws.total_tiles, st));
+      SV_TRY_CUDA(launch_tile_stage(c, tile_args(c, g, ws), mode, ws.search_all, ws.total_tiles, st));
       kt.done();
     }
     c->launches++;
-    finish_args(c, g, ws, mode);
+    finish_args(c, g, ws);
     {
       KTimer kt(c, kKStrag, st);
       SV_TRY_CUDA(launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st));
@@ -652,7 +654,7 @@ sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) 
 sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) {
   const uint32_t n = ws.n_reqs;
   const int mode = launch_mode(ws);
-  const sv_status bs = ensure_buffers(ws, g, mode);
+  const sv_status bs = ensure_buffers(ws, g);
   if (bs) return bs;
   ws.bucket_cap = g.bucket_cap;
   const bool init = n > kHostPlanMax;
@@ -666,7 +668,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
   static_assert(sizeof(ptrs) <= sizeof(key.p), "the key holds every pointer");
   std::memcpy(key.p, ptrs, sizeof(ptrs));
   key.g = g;
-  key.mode = (uint32_t)mode;
+  key.mode = (uint32_t)mode | (ws.ordered ? 16u : 0u);
   key.strag_cap = ws.strag_cap;
   key.search_all = ws.search_all ? 1u : 0u;
   key.n_class = range_class(n);
@@ -675,7 +677,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
   // per-kernel timing of the tile kernel: event-record nodes around it
   const bool timed = ((c->kprof >> ws.tile_kernel_id) & 1u) && st == c->stream;
   key.timed = timed ? 1u : 0u;
-  finish_args(c, g, ws, mode);
+  finish_args(c, g, ws);
   LaunchGraph *lg = nullptr;
   for (LaunchGraph &x : ws.graphs)
     if (x.exec && std::memcmp(&key, &x.key, sizeof(key)) == 0) lg = &x;
@@ -700,10 +702,10 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
     if (!e && c->n_primes > g.i_large)
       e = launch_bucket_fill(bucket_args(c, g, ws), c->n_primes - g.i_large, 1u << 20, 1ull << 23, fill_blocks(c), st);
     if (!e && timed) e = cudaEventRecordWithFlags(lg->ev[0], st, cudaEventRecordExternal);
-    if (!e) e = launch_tile_stage(c, tile_args(c, g, ws, mode), mode, ws.search_all, 0xFFFFFFFFu, st);
+    if (!e) e = launch_tile_stage(c, tile_args(c, g, ws), mode, ws.search_all, 0xFFFFFFFFu, st);
     if (!e && timed) e = cudaEventRecordWithFlags(lg->ev[1], st, cudaEventRecordExternal);
     if (!e && !ws.lazy_strag) e = launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st);
-    if (!e && mode == 0) e = launch_compact(ws.compact_args, 4u * (uint32_t)c->num_sms, st);  // grid-stride
+    if (!e && ws.ordered) e = launch_compact(ws.compact_args, 4u * (uint32_t)c->num_sms, st);  // grid-stride
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(st, &graph);
     if (e || e2 != cudaSuccess) {
@@ -755,7 +757,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
   // the graph reads the staging when it runs: the next plan waits for it
   if (!ws.staged && cudaEventCreateWithFlags(&ws.staged, cudaEventDisableTiming) != cudaSuccess) return SV_ECUDA;
   SV_TRY_CUDA(cudaEventRecord(ws.staged, st));
-  c->launches += 1u + (init ? 1u : 0u) + (c->n_primes > g.i_large ? 1u : 0u) + (ws.lazy_strag ? 0u : 1u) + (mode == 0 ? 1u : 0u);
+  c->launches += 1u + (init ? 1u : 0u) + (c->n_primes > g.i_large ? 1u : 0u) + (ws.lazy_strag ? 0u : 1u) + (ws.ordered ? 1u : 0u);
   ws.h2d_bytes = in_bytes;
   return SV_OK;
 }

@@ -180,7 +180,8 @@ struct TileArgs {
   uint32_t strag_cap;
   uint32_t *bucket_count;  // read, then cleared for the next launch
   const uint32_t *bucket_data;
-  // mode 0: tile t stages its list entries at [t * kStageCap, + stage_cnt[t])
+  // ordered lists (mode 0, and mode 2 unless null): tile t stages its list
+  // entries at [t * kStageCap, + stage_cnt[t])
   uint64_t *stage_n;
   uint8_t *stage_k;
   uint32_t *stage_cnt;
