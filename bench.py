@@ -81,9 +81,11 @@ def alu_ops_per_odd_n(hi: int) -> float:
 
 def strikes_per_launch(lo: int, hi: int, cfg) -> float:
     """Shared-memory atomics of one tile-kernel launch (algorithmic): every
-    window of 32 (tw + mw) bits takes window_bits / p^2 strikes of each prime
-    p >= 13 up to isqrt(hi - 1) (the stamped primes 3..11 are patterns, not
-    atomics)."""
+    window takes window_bits / p^2 strikes of each prime p >= 13 up to
+    isqrt(hi - 1) (the stamped primes 3..11 are patterns, not atomics).  A window
+    of the stream layout is 32 streams of 36 words per thread (a thread per 2^10
+    odd n of the tile knob), its margin a multiple of 9 words; other shapes take
+    the linear layout's 2^tile_log2 bits and margin."""
     import numpy as np
     lim = math.isqrt(hi - 1)
     sieve = np.ones(lim + 1, dtype=bool)
@@ -94,6 +96,10 @@ def strikes_per_launch(lo: int, hi: int, cfg) -> float:
     ps = np.nonzero(sieve)[0]
     ps = ps[ps >= 13].astype(np.float64)
     tw, mw = 1 << (cfg.tile_log2 - 5), 1 << (cfg.margin_log2 - 6)
+    threads = getattr(cfg, "threads", 0) or 512
+    if threads == 1 << (cfg.tile_log2 - 10) and (getattr(cfg, "stamp_primes", 0) or 4) == 4 and 15 <= cfg.tile_log2 <= 19:
+        mw = -(-mw // 9) * 9
+        tw = 36 * threads - mw
     jlo, jhi = (max(lo, 3) | 1) // 2, hi // 2
     words = (jhi + 31) // 32 - jlo // 32
     tiles = -(-words // tw)
@@ -157,7 +163,7 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-TILE_SOURCES = ("tiles.cu", "strike.h")  # the tile kernel's own source files
+TILE_SOURCES = ("streams.cu", "strike.h")  # the tile kernel's own source files
 
 
 def tile_source_sha() -> str:
@@ -306,7 +312,7 @@ def bench_range(name: str, stream, flush, steps: int, pk: dict, knobs: dict) -> 
     return {"workload": WORKLOAD_NAMES[name], "lo": lo, "hi": hi, "odd_n": n_odd, "steps": steps,
             "ms_per_step": ms, "value": n_odd / (ms / 1e3), "unit": UNIT,
             "roofline": {"bound": "alu", "achieved": achieved, "peak": pk["scan_mix_ops_per_s"], "unit": "int32 ops/s",
-                         "frac": achieved / pk["scan_mix_ops_per_s"], "kernel": "tile_kernel (sieve + scan, fused)",
+                         "frac": achieved / pk["scan_mix_ops_per_s"], "kernel": "stream_kernel (sieve + scan, fused)",
                          "kernel_avg_ms": tile_s * 1e3, "smem_atomic_frac": strikes / tile_s / pk["smem_atomic_strike_per_s"],
                          "peak_source": "measured in this run (sv_measure_peaks)"},
             "e2e": {"value": n_odd * e2e_steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d // e2e_steps,
@@ -692,7 +698,7 @@ def main() -> int:
                    "large_prime_min": v.config.large_prime_min, "stamp_primes": v.config.stamp_primes},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak, "unit": "int32 ops/s",
                      "frac": achieved / alu_peak, "traffic": measured_traffic(n_odd),
-                     "kernel": "tile_kernel (sieve + scan, fused)",
+                     "kernel": "stream_kernel (sieve + scan, fused)",
                      "peak_source": "measured in this run: sv_measure_peaks, the scan's integer mix "
                                     "(funnel shift, AND-NOT, popcount, add) on every SM",
                      "ops_per_odd_n": ops_per_n, "kernel_avg_ms": tile_avg_s * 1e3,

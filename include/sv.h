@@ -69,7 +69,8 @@ typedef struct sv_ctx sv_ctx; /* opaque: prime table, scratch, streams, graphs, 
  * changes any result; they only change speed and memory.
  */
 typedef struct sv_config {
-    uint32_t tile_log2;          /* odd numbers per shared-memory tile = 2^tile_log2 (14..20) */
+    uint32_t tile_log2;          /* odd numbers per shared-memory tile = 2^tile_log2 (14..20), or nearly so;
+                                    launches of few tiles take smaller ones */
     uint32_t margin_log2;        /* look-back below each tile, in integers: W = 2^margin_log2
                                     (6..tile_log2+1).  n - 2^k with 2^k <= W is read from the
                                     tile's own window; larger k go to the exact straggler test */

@@ -1,5 +1,13 @@
-// tiles.cu -- the range path: Algorithm 1 (sieve) and Algorithm 2 (search
-// for the smallest k) of Sec. 3, fused per shared-memory tile.
+// tiles.cu -- the linear layout: Algorithm 1 (sieve) and Algorithm 2 (search
+// for the smallest k) of Sec. 3, fused per shared-memory tile, with one bit
+// per odd n in the order of n.
+//
+// Launches of aggregates and ordered lists run in the stream layout
+// (streams.cu), which does the same work on 2^33 odd n in 398 us against 601
+// here.  This layout serves what that one has no form for: the per-n output,
+// whose bytes leave in the order of n; the bitmap, and the plain path's two
+// passes; lists with T < 6 and unordered lists; and block shapes or windows
+// without a stream counterpart.
 //
 // Persistent CTAs (two per SM by default) take chunks of consecutive tiles
 // from a device work counter.  A tile is 2^tile_log2 consecutive odd numbers
