@@ -1388,11 +1388,12 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
       free_table();
       return SV_ENOMEM;
     }
-    c->d_stamp = d_stamp;
     if (launch_stamp_tables(d_stamp, c->stream) != cudaSuccess) {
+      cudaFree(d_stamp);
       free_table();
       return SV_ECUDA;
     }
+    c->d_stamp = d_stamp;
     c->launches += kStreamSizes;
   }
   std::vector<uint32_t> hp(n);

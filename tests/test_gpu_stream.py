@@ -59,3 +59,19 @@ def test_batches_of_short_ranges(gpu, orc):
     res = gpu.verify_batch([a for a, _ in reqs], [b for _, b in reqs])
     for g, o in zip(res, orc.verify_ranges(reqs)):
         assert_same_range(g, o, per_n=False)
+
+
+@pytest.mark.parametrize("n,k,margin", [(60690478781437, 13, 12), (9579717479644589, 14, 13)])
+def test_an_n_beyond_the_look_back(orc, n, k, margin):
+    # a look-back of 2^12 or more: the exact test of the n beyond it is
+    # launched only after the results have counted one
+    rng = (n - 40000, n + 60000)
+    o = orc.verify_range(*rng)
+    assert o.hist[k] == 1 and o.first_n[k] == n
+    with Verifier(max_hi=1 << (n.bit_length() + 1), margin_log2=margin) as v:
+        assert_same_range(v.verify_range(*rng), o, per_n=False)
+        v.launch_range(*rng)
+        assert_same_range(v.fetch_range(), o, per_n=False)
+        for count in (3, 40):
+            for g in v.verify_batch([rng[0]] * count, [rng[1]] * count):
+                assert_same_range(g, o, per_n=False)
