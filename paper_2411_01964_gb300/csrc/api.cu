@@ -157,7 +157,8 @@ Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges 
   Geometry g{};
   g.tw = 1u << (k.tile_log2 - shrink - 5);
   g.mw = 1u << (k.margin_log2 - 6);
-  g.threads = std::max(k.threads >> shrink, std::min(k.threads, kLinearMinThreads));
+  // (whole warps: the knob is any multiple of 32, and half of 544 is not one)
+  g.threads = std::max((k.threads >> shrink) & ~31u, std::min(k.threads, kLinearMinThreads));
   g.ctas = std::min(k.ctas_per_sm * (k.threads / g.threads), std::max(k.ctas_per_sm, 4u));
   if (stream_threads) {
     g.stream = 1;
