@@ -421,6 +421,10 @@ sv_status sv_measure_peaks(sv_ctx *ctx, sv_peaks *out);
  */
 sv_status sv_inject_alloc_failures(sv_ctx *ctx, uint32_t count);
 
+/* The same after `skip` further allocations that succeed, so that a chosen one
+ * of several buffers that grow together fails. */
+sv_status sv_inject_alloc_failures_after(sv_ctx *ctx, uint32_t skip, uint32_t count);
+
 /*
  * Test hook for the bounded waits: the next `count` plain-path launches of
  * this context (sv_verify_range_plain, sv_launch_range_plain) leave out their

@@ -19,7 +19,7 @@ using namespace sv;
 
 namespace sv {
 
-std::atomic<uint32_t> g_inject_alloc_failures{0};
+std::atomic<uint32_t> g_inject_alloc_failures{0}, g_inject_alloc_skip{0};
 
 void Workspace::release_all() {
   for (LaunchGraph &lg : graphs) {
@@ -474,11 +474,11 @@ bool ensure_stage(Workspace &ws) {
 // The device buffers of the planned launch.
 sv_status ensure_buffers(Workspace &ws, const Geometry &g) {
   const size_t tiles = ws.total_tiles ? ws.total_tiles : 1;
-  const size_t counts = ws.bucket_count.cap;
+  // (the counts grow, perhaps in place: no longer clear, also if an allocation after them fails)
+  if (tiles > ws.bucket_count.cap) ws.counts_clean = false;
   if (ws.fail_n.ensure(ws.fail_total ? ws.fail_total : 1) || ws.strag.ensure(ws.strag_cap) ||
       ws.bucket_count.ensure(tiles) || ws.bucket_data.ensure(tiles * g.bucket_cap))
     return SV_ENOMEM;
-  if (ws.bucket_count.cap != counts) ws.counts_clean = false;  // grown (perhaps in place)
   if (ws.ordered && !ensure_stage(ws)) return SV_ENOMEM;
   return SV_OK;
 }
@@ -1736,7 +1736,13 @@ sv_status sv_inject_bulk_timeout(sv_ctx *c, uint32_t count) {
 }
 
 sv_status sv_inject_alloc_failures(sv_ctx *c, uint32_t count) {
+  return sv_inject_alloc_failures_after(c, 0, count);
+}
+
+sv_status sv_inject_alloc_failures_after(sv_ctx *c, uint32_t skip, uint32_t count) {
   if (!c) return SV_EINVAL;
+  g_inject_alloc_failures.store(0);
+  g_inject_alloc_skip.store(skip);
   g_inject_alloc_failures.store(count);
   return SV_OK;
 }

@@ -15,11 +15,15 @@ namespace sv {
 
 constexpr int kPiBlockLog2 = 12;  // block size of the host prime-count index
 
-// Allocations still to fail on purpose (sv_inject_alloc_failures); takes one
-// if any is left.
-extern std::atomic<uint32_t> g_inject_alloc_failures;
+// Allocations still to fail on purpose (sv_inject_alloc_failures) and those to
+// let through before them; takes a failure if one is due.
+extern std::atomic<uint32_t> g_inject_alloc_failures, g_inject_alloc_skip;
 inline bool take_injected_failure() {
   uint32_t n = g_inject_alloc_failures.load();
+  if (n == 0) return false;
+  uint32_t skip = g_inject_alloc_skip.load();
+  while (skip > 0)
+    if (g_inject_alloc_skip.compare_exchange_weak(skip, skip - 1)) return false;
   while (n > 0 && !g_inject_alloc_failures.compare_exchange_weak(n, n - 1)) {
   }
   return n > 0;
