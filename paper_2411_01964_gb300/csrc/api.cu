@@ -887,12 +887,14 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
   // one range whose caller buffers are pinned host memory: its list region
   // goes straight into them (no staging copy, no host copy afterwards); the
   // entries past the list's length are left unspecified
-  bool direct = false;
+  bool direct = spec_end && n == 1 && outs[0] && is_pinned(outs[0]->list) && is_pinned(outs[0]->list_k);
   uint64_t direct_m = 0;
+  // (before any copy is enqueued: a copy left behind by a failed call would
+  // land in the staging while the next call plans in it)
+  if (spec_end && !direct && (ws.h_list_n.ensure(spec_end) || ws.h_list_k.ensure(spec_end))) return SV_ENOMEM;
   for (;;) {
     SV_TRY_CUDA(cudaMemcpyAsync(ws.h_io.p + ws.io_hdr, ws.io.p + ws.io_hdr, out_bytes, cudaMemcpyDeviceToHost, st));
-    if (spec_end && n == 1 && outs[0] && is_pinned(outs[0]->list) && is_pinned(outs[0]->list_k)) {
-      direct = true;
+    if (direct) {
       direct_m = std::min<uint64_t>(ws.h_reqs[0].list_cap, outs[0]->list_cap);
       const uint64_t off = ws.h_reqs[0].list_off;
       if (direct_m && outs[0]->list)
@@ -900,7 +902,6 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
       if (direct_m && outs[0]->list_k)
         SV_TRY_CUDA(cudaMemcpyAsync(outs[0]->list_k, ws.d_list_k + off, direct_m, cudaMemcpyDeviceToHost, st));
     } else if (spec_end) {
-      if (ws.h_list_n.ensure(spec_end) || ws.h_list_k.ensure(spec_end)) return SV_ENOMEM;
       SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_n.p, ws.d_list_n, 8 * spec_end, cudaMemcpyDeviceToHost, st));
       SV_TRY_CUDA(cudaMemcpyAsync(ws.h_list_k.p, ws.d_list_k, spec_end, cudaMemcpyDeviceToHost, st));
     }

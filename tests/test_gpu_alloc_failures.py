@@ -49,3 +49,23 @@ def test_bucket_counts_grown_before_the_buckets_fail(orc):
         for _ in range(2):
             bits, f0, cnt = unpack_bitmap(v.sieve_bitmap(lo, short).cpu().numpy().view(np.uint32), lo, short)
             assert np.array_equal(bits[f0:f0 + cnt], want)
+
+
+@pytest.mark.parametrize("skip", range(10))
+def test_any_allocation_of_a_growing_call(orc, skip):
+    # whichever buffer fails, a call that fits the buffers of before is exact
+    lo = (1 << 44) + 12345
+    small, large = lo + (1 << 22), lo + (1 << 30)
+    o = orc.verify_range(lo, small)
+    with Verifier(max_hi=1 << 45) as v:
+        assert v.verify_range(lo, small).hist == o.hist
+        B.sv_inject_alloc_failures_after(v.ctx, skip, 1)
+        try:
+            v.verify_range(lo, large)
+        except B.SvError as e:
+            assert e.status == B.SV_ENOMEM
+        B.sv_inject_alloc_failures(v.ctx, 0)
+        for hi in (small, lo + (1 << 24)):
+            o = orc.verify_range(lo, hi)
+            g = v.verify_range(lo, hi)
+            assert g.hist == o.hist and g.first_n == o.first_n and np.array_equal(g.list_n, o.list_n)
