@@ -381,6 +381,9 @@ class Server {
     if (s.npoints) st = launch_points_async(c_, s.npoints, s.ws, s.st);
     if (!st && !s.items.empty()) st = launch_ranges_async(c_, s.specs, s.ws, s.st);
     if (cudaEventRecord(s.ev, s.st) != cudaSuccess && !st) st = SV_ECUDA;
+    // what was enqueued before a failure still reads the slot's staging, which
+    // the slot's next work overwrites
+    if (st) cudaStreamSynchronize(s.st);
     return st;
   }
 

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2411_01964_gb300 import B, Verifier
+from paper_2411_01964_gb300 import B, Verifier, inputs
 from test_gpu_parity import unpack_bitmap
 
 pytestmark = pytest.mark.gpu
@@ -69,3 +69,24 @@ def test_any_allocation_of_a_growing_call(orc, skip):
             o = orc.verify_range(lo, hi)
             g = v.verify_range(lo, hi)
             assert g.hist == o.hist and g.first_n == o.first_n and np.array_equal(g.list_n, o.list_n)
+
+
+def test_points_of_a_launch_whose_ranges_fail(orc):
+    # the points of a slot are launched first; when its ranges then fail for
+    # want of memory, the slot's next points are answered from their own staging
+    lo = (1 << 44) + 12345
+    with Verifier(max_hi=1 << 46, serve_slots=1) as v:
+        t = v.submit_points([3])
+        assert v.poll(t, -1) == B.SV_OK
+        for i, count in enumerate((2048, 1024, 40000, 2048)):
+            B.sv_inject_alloc_failures(v.ctx, 1 << 20)
+            burst = [v.prepare_points(inputs.random_points(10 + i, count, 2, 1 << 44)),
+                     v.prepare_range(lo, lo + (1 << 24))]
+            v.submit_many(burst)
+            assert v.poll(burst[1], -1) == B.SV_ENOMEM
+            B.sv_inject_alloc_failures(v.ctx, 0)
+            pts = inputs.random_points(20 + i, 1500, 2, 1 << 44)
+            after = v.submit_points(pts)
+            v.poll(burst[0], -1)
+            assert v.poll(after, -1) == B.SV_OK
+            assert np.array_equal(after.result(), orc.min_k(pts))
