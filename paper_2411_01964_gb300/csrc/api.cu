@@ -664,7 +664,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
   GraphKey key;
   std::memset(&key, 0, sizeof(key));
   const void *ptrs[] = {ws.io.p,      ws.h_io.p,  ws.slots,          ws.d_list_n,        ws.d_list_k,
-                        ws.fail_n.p,  ws.strag.p, ws.bucket_count.p, ws.bucket_data.p,   c->d_p,
+                        ws.fail_n.p,  ws.strag.p, ws.bucket_count.p, ws.bucket_data.p,
                         (const void *)st, ws.stage_n.p, ws.stage_k.p, ws.stage_cnt.p};
   static_assert(sizeof(ptrs) <= sizeof(key.p), "the key holds every pointer");
   std::memcpy(key.p, ptrs, sizeof(ptrs));
@@ -674,7 +674,7 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
   key.search_all = ws.search_all ? 1u : 0u;
   key.n_class = range_class(n);
   key.in_bytes = in_bytes;
-  key.n_table = c->n_primes;
+  key.table_id = c->table_id;
   // per-kernel timing of the tile kernel: event-record nodes around it
   const bool timed = ((c->kprof >> ws.tile_kernel_id) & 1u) && st == c->stream;
   key.timed = timed ? 1u : 0u;
@@ -907,8 +907,10 @@ sv_status collect(sv_ctx *c, const std::vector<RangeSpec> &specs, sv_range_resul
     }
     SV_TRY_CUDA(cudaStreamSynchronize(st));
     if (!ws.lazy_strag || !ws.h_hdr->strag_count || ws.h_hdr->status) break;
-    // stragglers after all: their kernel, the lists again, and another look
+    // stragglers after all: their kernel (with today's prime table: the
+    // launch's may have been replaced), the lists again, and another look
     ws.lazy_strag = false;
+    ws.strag_args.pt = prime_tab(c);
     SV_TRY_CUDA(launch_stragglers(ws.strag_args, (uint32_t)c->num_sms * 2, st));
     c->launches++;
     if (ws.compact_grid) {
@@ -1404,12 +1406,20 @@ sv_status sv_init_primes(sv_ctx *c, uint64_t max_hi) {
     return SV_ECUDA;
   }
   cudaStreamSynchronize(c->stream);
+  // launches in flight read the old table until they end; what is left to be
+  // launched for them (collect) takes the new one
+  std::lock_guard<std::mutex> tl(c->table_mu);
+  if (c->server && cudaDeviceSynchronize() != cudaSuccess) {
+    free_table();
+    return SV_ECUDA;
+  }
   cudaFree(c->d_p);
   cudaFree(c->d_mu);
   cudaFree(c->d_inv);
   cudaFree(c->d_lim);
   cudaFree(c->d_pbits);
   cudaFree(c->d_word);
+  ++c->table_id;
   c->d_word = d_word;
   c->d_p = d_p;
   c->d_mu = d_mu;

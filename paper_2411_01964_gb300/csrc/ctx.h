@@ -81,8 +81,8 @@ struct GraphKey {
   Geometry g;
   uint32_t mode, strag_cap, search_all, n_class;
   uint64_t in_bytes;
-  uint32_t n_table;
-  uint32_t timed;  // 1: event-record nodes bracket the tile kernel
+  uint64_t table_id;  // the prime table (its arrays' addresses may be used again)
+  uint64_t timed;     // 1: event-record nodes bracket the tile kernel
 };
 
 // A captured launch graph and what it was captured for; a timed graph keeps
@@ -191,7 +191,10 @@ struct sv_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::mutex mu;            // serialises the blocking / device-resident calls
-  // prime table
+  // prime table; replaced under mu and table_mu, read under either (the
+  // serving thread holds table_mu)
+  std::mutex table_mu;
+  uint64_t table_id = 0;    // counts the tables
   uint64_t max_hi = 0, pmax = 0;
   uint32_t *d_p = nullptr;
   uint64_t *d_mu = nullptr, *d_inv = nullptr, *d_lim = nullptr;

@@ -377,6 +377,7 @@ class Server {
     // the points first: behind the ranges they would wait for room until the
     // next slot's tile kernel, which fills the GPU meanwhile, is done, and this
     // slot's results with them
+    std::lock_guard<std::mutex> tl(c_->table_mu);
     sv_status st = SV_OK;
     if (s.npoints) st = launch_points_async(c_, s.npoints, s.ws, s.st);
     if (!st && !s.items.empty()) st = launch_ranges_async(c_, s.specs, s.ws, s.st);
@@ -413,6 +414,7 @@ class Server {
       ptrs[i] = &o;
     }
     if (!st && n) {
+      std::lock_guard<std::mutex> tl(c_->table_mu);  // the launch may have to be completed or repeated
       bool retry = false;
       st = collect_ranges(c_, s.specs, ptrs.data(), s.ws, s.st, &retry);
       if (!st && retry) {
