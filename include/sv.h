@@ -422,7 +422,9 @@ sv_status sv_measure_peaks(sv_ctx *ctx, sv_peaks *out);
 sv_status sv_inject_alloc_failures(sv_ctx *ctx, uint32_t count);
 
 /* The same after `skip` further allocations that succeed, so that a chosen one
- * of several buffers that grow together fails. */
+ * of several buffers that grow together fails.  The contents of a fresh device
+ * allocation are unspecified; while failures are due, every one is filled with
+ * bytes of 1. */
 sv_status sv_inject_alloc_failures_after(sv_ctx *ctx, uint32_t skip, uint32_t count);
 
 /*

@@ -47,6 +47,11 @@ struct Buf {
       return e;
     }
     cap = c;
+    // the test hook: nothing may rely on what a fresh allocation holds
+    if (!PINNED && g_inject_alloc_failures.load()) {
+      cudaMemset(p, 1, c * sizeof(T));
+      cudaStreamSynchronize(cudaStreamLegacy);
+    }
     return cudaSuccess;
   }
   void release() {

@@ -3,7 +3,6 @@ the host): the call returns SV_ENOMEM, and the next calls on the same context
 are exact.  Integers: equality with the CPU oracle."""
 import numpy as np
 import pytest
-import torch
 
 from paper_2411_01964_gb300 import B, Verifier, inputs
 from test_gpu_parity import unpack_bitmap
@@ -24,31 +23,23 @@ def enomem(call):
     assert e.value.status == B.SV_ENOMEM
 
 
-def used_device_memory(value):
-    """Leaves `value` in device memory that the next allocations may get."""
-    keep = [torch.full((n,), value, dtype=torch.int32, device="cuda") for n in (1 << 19, 1 << 20, 1 << 21, 1 << 24)]
-    torch.cuda.synchronize()
-    del keep
-    torch.cuda.empty_cache()
-
-
 def test_bucket_counts_grown_before_the_buckets_fail(orc):
-    # tiles of 2^14 odd n with a margin of 32 bits and buckets of 1024 entries:
-    # a stale count of 40 would strike bit 40 of every tile, which its output shows
+    # stale counts would fill the buckets up: wrong strikes, or a launch repeated with deeper buckets
     lo = (1 << 40) + 64
-    short, long = lo + (1 << 21), lo + (1 << 34)  # 64 tiles; 2^19 + 1, whose counts are an allocation of their own
-    with Verifier(max_hi=1 << 41, tile_log2=14, margin_log2=6, bucket_capacity=1024) as v:
-        bits, f0, cnt = unpack_bitmap(v.sieve_bitmap(lo, short).cpu().numpy().view(np.uint32), lo, short)
-        want = orc.sieve_odd(lo, short)
-        assert np.array_equal(bits[f0:f0 + cnt], want)
-        room = torch.empty(B.sv_bitmap_words(lo, long), dtype=torch.int32, device="cuda")
-        used_device_memory(40)
-        B.sv_inject_alloc_failures_after(v.ctx, 1, 1)  # the counts grow, the buckets do not
-        enomem(lambda: B.check(B.sv_sieve_bitmap(v.ctx, lo, long, room.data_ptr()), "sv_sieve_bitmap"))
-        B.sv_inject_alloc_failures(v.ctx, 0)
-        for _ in range(2):
+    short, long = lo + (1 << 21), lo + (1 << 24)
+    want = orc.sieve_odd(lo, short)
+    with Verifier(max_hi=1 << 41, tile_log2=14, margin_log2=6) as v:
+        def bitmap_is_exact():
+            before = v.kernel_launches()
             bits, f0, cnt = unpack_bitmap(v.sieve_bitmap(lo, short).cpu().numpy().view(np.uint32), lo, short)
             assert np.array_equal(bits[f0:f0 + cnt], want)
+            return v.kernel_launches() - before
+
+        launches = bitmap_is_exact()
+        B.sv_inject_alloc_failures_after(v.ctx, 1, 1)  # the counts grow, the buckets do not
+        enomem(lambda: v.sieve_bitmap(lo, long))
+        B.sv_inject_alloc_failures(v.ctx, 0)
+        assert bitmap_is_exact() == launches
 
 
 @pytest.mark.parametrize("skip", range(10))
