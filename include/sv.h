@@ -444,8 +444,8 @@ uint64_t sv_kernel_launches(const sv_ctx *ctx);
  * bracketed by CUDA events recorded on the stream it is launched on.  A
  * launch replayed from a captured graph times only its tile kernel (id 2),
  * through event-record nodes given fresh events at every replay; the others
- * in it are not timed, so sv_launch_range takes the graph path only while no
- * other kernel is timed.  enable: 0 off, -1 every
+ * in it are not timed, so sv_launch_range and sv_sieve_bitmap take the graph
+ * path only while no other kernel is timed.  enable: 0 off, -1 every
  * kernel, otherwise a bit mask of kernel ids (bit i: id i); every call resets
  * the totals.  Kernel ids: 0 init, 1 bucket fill, 2 tile (sieve + scan),
  * 3 stragglers, 4 points, 5 ordered-list compaction, 6 tile kernel of the

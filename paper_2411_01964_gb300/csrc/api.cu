@@ -591,6 +591,10 @@ struct KTimer {
   }
 };
 
+// A launch may be a captured graph (fewer launch gaps) unless a kernel other
+// than the tile kernel is being timed: a graph brackets only the tile kernel.
+bool graph_can_time(const sv_ctx *c) { return (c->kprof & ~(1u << c->ws.tile_kernel_id)) == 0; }
+
 // Enqueues init -> bucket fill -> tiles -> stragglers for the planned launch.
 sv_status enqueue(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_t st) {
   const uint32_t n = ws.n_reqs;
@@ -1612,7 +1616,7 @@ sv_status sv_sieve_bitmap(sv_ctx *c, uint64_t lo, uint64_t hi, uint32_t *d_bitma
   specs[0].hi = hi;
   specs[0].sieve_only = true;
   specs[0].bitmap_out = d_bitmap;
-  return run_ranges(c, specs, nullptr, c->stream, c->ws, true);
+  return run_ranges(c, specs, nullptr, c->stream, c->ws, graph_can_time(c));
 }
 
 sv_status sv_launch_range(sv_ctx *c, uint64_t lo, uint64_t hi, uint8_t *d_per_n_k) {
@@ -1630,10 +1634,7 @@ sv_status sv_launch_range(sv_ctx *c, uint64_t lo, uint64_t hi, uint8_t *d_per_n_
   specs[0].fail_cap = 1024;
   const Geometry g = geometry_of(c, specs, c->ws);
   if ((s = plan(c, specs, g, c->ws))) return s;
-  // the captured graph (fewer launch gaps), unless a kernel other than the
-  // tile kernel is being timed: a graph brackets only the tile kernel
-  const bool graph = (c->kprof & ~(1u << c->ws.tile_kernel_id)) == 0;
-  if ((s = graph ? enqueue_graph(c, g, c->ws, c->stream) : enqueue(c, g, c->ws, c->stream))) return s;
+  if ((s = graph_can_time(c) ? enqueue_graph(c, g, c->ws, c->stream) : enqueue(c, g, c->ws, c->stream))) return s;
   c->pending = true;
   c->pending_plain = false;
   c->pending_specs = specs;
