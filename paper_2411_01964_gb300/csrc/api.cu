@@ -1616,7 +1616,9 @@ sv_status sv_sieve_bitmap(sv_ctx *c, uint64_t lo, uint64_t hi, uint32_t *d_bitma
   specs[0].hi = hi;
   specs[0].sieve_only = true;
   specs[0].bitmap_out = d_bitmap;
-  return run_ranges(c, specs, nullptr, c->stream, c->ws, graph_can_time(c));
+  // (the legacy default stream cannot be captured)
+  const bool graph = graph_can_time(c) && c->stream != cudaStreamLegacy;
+  return run_ranges(c, specs, nullptr, c->stream, c->ws, graph);
 }
 
 sv_status sv_launch_range(sv_ctx *c, uint64_t lo, uint64_t hi, uint8_t *d_per_n_k) {

@@ -1,5 +1,6 @@
 """sv_sieve_bitmap beside its captured graph: the timing of other kernels than
-the tile kernel."""
+the tile kernel, and a context on the legacy default stream, which cannot be
+captured."""
 import numpy as np
 import pytest
 
@@ -26,3 +27,9 @@ def test_timed_kernels(orc, kernels):
         for name, i in B.KERNEL_IDS.items():
             ms, n = B.sv_kernel_time(v.ctx, i)
             assert n == (name in kernels) and (ms > 0) == (name in kernels)
+
+
+def test_legacy_stream(orc):
+    with Verifier(max_hi=1 << 41, stream=1) as v:
+        assert_bitmap(v, orc)
+        assert_bitmap(v, orc)
