@@ -101,7 +101,13 @@ struct LaunchGraph {
   cudaEvent_t ev[2] = {nullptr, nullptr};  // the events recorded at capture
   uint64_t used = 0;                       // the launch that used it last
 };
-constexpr int kGraphs = 4;  // graphs kept per workspace: launches of a few shapes alternate without capturing anew
+// Graphs kept per workspace, so that launches of several shapes alternate
+// without capturing anew: short ranges in batches of 1 to 32 at random have six
+// layouts (range_class), single ranges of any length four block sizes and as
+// many bucket thresholds.  Batches of 1 to 32: 61 to 63 us a call with four
+// graphs, 56 with eight; calls of single ranges, bitmaps and batches in turn 60
+// and 53.
+constexpr int kGraphs = 8;
 
 // Everything one launch needs on the device, reused across launches.
 struct Workspace {
