@@ -6,6 +6,7 @@
 #include <atomic>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "sv.h"
@@ -89,6 +90,7 @@ struct GraphKey {
   uint64_t table_id;  // the prime table (its arrays' addresses may be used again)
   uint64_t timed;     // 1: event-record nodes bracket the tile kernel
 };
+static_assert(std::has_unique_object_representations_v<GraphKey>, "no padding, whose bytes nothing sets");
 
 // A captured launch graph and what it was captured for; a timed graph keeps
 // its event-record nodes around the tile kernel (node), whose events are

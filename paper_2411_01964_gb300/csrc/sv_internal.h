@@ -151,9 +151,9 @@ struct Geometry {
   uint32_t stage_cap; // usable staged list entries per tile (<= kStageCap)
   uint32_t threads;   // threads per block of the tile kernel
   uint32_t ctas;      // its resident blocks per SM
-  uint32_t pad;
   uint64_t tw_inv;    // floor((2^64 - 1) / tw), for tile_index
 };
+static_assert(sizeof(Geometry) == 16 * sizeof(uint32_t) + sizeof(uint64_t), "no padding: compared bytewise (GraphKey)");
 
 // The tile holding the dw-th word of a range: dw / tw (the estimate is at
 // most one low for dw < 2^63).
