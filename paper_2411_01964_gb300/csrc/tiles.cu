@@ -21,7 +21,7 @@
 //   2. strike: the next primes up to the bucket threshold clear their odd
 //              multiples of p^2 with shared-memory atomicAnd.  "Dense" primes
 //              (>= kDenseMinHits hits per window, at most 128) are struck
-//              cooperatively, two strikes per trip:
+//              cooperatively, each thread with one mask per prime:
 //              the smallest by the whole CTA with a stride of one block, the
 //              others by one warp each with a stride of one warp.  Sparser
 //              ones take one thread per prime.  The offsets of both carry
@@ -1133,6 +1133,10 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(TileArgs a) {
 
 static bool g_tile_smem_set = false;
 
+// An upper bound of the tile kernel's static shared memory (all
+// instantiations: mode 2 has the per-n table of 256 words).
+size_t tile_static_smem() { return sizeof(ScanShared) + 4 * StampTab<8>::kSize + 4 * 256 + 256; }
+
 // Raise one instantiation's dynamic shared memory limit to what its static
 // shared memory leaves of the opt-in limit.
 template <class K>
@@ -1140,6 +1144,7 @@ static cudaError_t set_max_dyn(K kernel, int optin) {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
+  if (fa.sharedSizeBytes > tile_static_smem()) return cudaErrorInvalidConfiguration;  // the bound is to be one
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
@@ -1162,9 +1167,6 @@ cudaError_t tile_kernel_setup(size_t smem) {
   g_tile_smem_set = true;
   return cudaSuccess;
 }
-
-// An upper bound of the tile kernel's static shared memory (all instantiations).
-size_t tile_static_smem() { return sizeof(ScanShared) + 4 * StampTab<8>::kSize + 256; }
 
 cudaError_t launch_tiles(const TileArgs &a, uint32_t threads, uint32_t grid, size_t smem, int mode, cudaStream_t st) {
   if (grid == 0) return cudaSuccess;
