@@ -505,9 +505,10 @@ __device__ __forceinline__ void scan_tile_lean(const uint32_t *win, const TileAr
       SV_DEFER(I1, u1)                                                              \
     }                                                                               \
   }
-  if (need == 0u && ifl <= mw && nfull >= nwords - ifl && (nwords - mw) % (64u * nwarps) == 0u) {
+  if (need == 0u && ifl <= mw && nfull >= nwords - ifl && (nwords - mw) % (64u * nwarps) == 0u && (mw & 1u) == 0u) {
     // every core word is in range and fully valid, and no first occurrence
-    // is searched: no masks, no bounds checks.  Each warp scans one
+    // is searched: no masks, no bounds checks.  (A margin of one word would
+    // leave the 64-bit loads misaligned.)  Each warp scans one
     // contiguous span, 64 words per step: lane l loads words 2l and 2l + 1
     // at once; the word below 2l is lane l-1's second word (lane 0: the
     // previous step's last word).
