@@ -315,15 +315,18 @@ struct ScanShared {
 // load; the outcome is the same for every thread of the block.
 constexpr long long kBulkWaitCycles = 2000000000ll;
 
-// Record the n of hit (mink = k, k >= T) in the range's list and first_n.
-__device__ __noinline__ void list_append(const TileArgs &a, const ReqDesc &R, uint32_t hit,
-                                         uint64_t J0, uint32_t k) {
+// Record the n of hit (mink = k, k >= T) in the range's list, and the first of
+// them in the tile's first occurrences (a global minimum per n doubled the time
+// of launches with long lists when first_n and list_count fell to one L2 slice:
+// 2^28 integers with T = 3 3906 us, with the two in different slices 2124).
+__device__ __noinline__ void list_append(const TileArgs &a, ScanShared &sh, uint32_t hit, uint64_t J0, uint32_t k) {
+  const ReqDesc &R = sh.req;
   ResultSlot *slot = &a.slots[R.slot];
+  atomicMin(&sh.first[k], (unsigned long long)(2ull * (J0 + (uint64_t)(__ffs(hit) - 1)) + 1ull));
   while (hit) {
     const uint32_t b = __ffs(hit) - 1;
     hit &= hit - 1;
     const uint64_t n = 2ull * (J0 + b) + 1ull;
-    atomicMin(&slot->first_n[k], (unsigned long long)n);
     const unsigned long long idx = atomicAdd(&slot->list_count, 1ull);
     if (idx < R.list_cap) {
       a.list_n[R.list_off + idx] = n;
@@ -383,7 +386,7 @@ __device__ __noinline__ void scan_tail(const uint32_t *win, uint32_t i, bool act
         atomicMin(&sh.first[k], (unsigned long long)(2ull * (J0 + (uint64_t)(__ffs(hit) - 1)) + 1ull));
       if (k >= rec_t) {
         if (LEAN) list_buffer(sh, hit, J0, k);
-        else list_append(a, sh.req, hit, J0, k);
+        else list_append(a, sh, hit, J0, k);
       }
     }
   }
@@ -421,7 +424,7 @@ __device__ __forceinline__ void scan_word(const uint32_t *win, uint32_t i, bool 
   unres &= ~(SF);                                               \
   if (!(LEAN && K == 1)) CNT += __popc(h);                      \
   if (REC) record_first<K>(h, need, sh, 32ull * (uint64_t)aw);                    \
-  if (!LEAN && (uint32_t)K >= rec_t && h) list_append(a, sh.req, h, 32ull * (uint64_t)aw, (uint32_t)K);
+  if (!LEAN && (uint32_t)K >= rec_t && h) list_append(a, sh, h, 32ull * (uint64_t)aw, (uint32_t)K);
   SV_STEP(1, __funnelshift_l(wp, w, 1), c1)
   if (__any_sync(0xFFFFFFFFu, unres)) {
     SV_STEP(2, __funnelshift_l(wp, w, 2), c2)
@@ -662,7 +665,7 @@ __device__ __noinline__ void finish_per_n(const uint32_t *win, int32_t P, uint32
     atomicMin(&sh.first[k], (unsigned long long)(2ull * (J + (uint64_t)(__ffs(h) - 1)) + 1ull));
     if (k >= rec_t) {
       if (a.stage_n) list_buffer(sh, h, J, k);  // an ordered list (T >= 6)
-      else list_append(a, sh.req, h, J, k);
+      else list_append(a, sh, h, J, k);
     }
     for (uint32_t m = h; m; m &= m - 1) out[__ffs(m) - 1] = (uint8_t)k;
   }
@@ -728,10 +731,10 @@ __device__ __forceinline__ void scan_tile_per_n(const uint32_t *win, const TileA
       record_first<4>(u3 & ~u4, need, sh, J);
     }
     if (rec_t <= 4) {
-      if (rec_t <= 1 && (valid & ~u1)) list_append(a, R, valid & ~u1, J, 1);
-      if (rec_t <= 2 && (u1 & ~u2)) list_append(a, R, u1 & ~u2, J, 2);
-      if (rec_t <= 3 && (u2 & ~u3)) list_append(a, R, u2 & ~u3, J, 3);
-      if (u3 & ~u4) list_append(a, R, u3 & ~u4, J, 4);
+      if (rec_t <= 1 && (valid & ~u1)) list_append(a, sh, valid & ~u1, J, 1);
+      if (rec_t <= 2 && (u1 & ~u2)) list_append(a, sh, u1 & ~u2, J, 2);
+      if (rec_t <= 3 && (u2 & ~u3)) list_append(a, sh, u2 & ~u3, J, 3);
+      if (u3 & ~u4) list_append(a, sh, u3 & ~u4, J, 4);
     }
     if (u4) finish_per_n(win, P, nwords, u4, J, o, a, sh);
     __syncwarp();
