@@ -252,17 +252,27 @@ uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, co
 }
 
 // How often a launch of the linear layout halves its tiles: until there are
-// two tiles per SM, or a tile holds 2^15 odd n, or its margin is an eighth of
-// it.  (2^24 integers are 16 tiles of 2^19 odd n, which leave 136 SMs idle: with
-// the per-n output 643 us a call, 306 in 256 tiles.)
+// three for every two SMs, or a tile holds 2^15 odd n, or its margin is an
+// eighth of it.  (2^24 integers are 16 tiles of 2^19 odd n, which leave 136 SMs
+// idle: with the per-n output 643 us a call, 306 in 256 tiles.  From three for
+// two SMs on, the halves come to four on some SM, as much as two whole tiles:
+// the per-n output of 2^28 integers, 257 tiles, 78 us whole and 90 halved, of
+// 220 * 2^20, 211 tiles, 78 and 68; lists with T = 5 57 and 77, 56 and 56.)
+// Lists with T <= 3 hold 2% of the n and more and are sorted by the host, which
+// scatters the entries of as many tiles as arrive together: sixteen then (all
+// odd n of 2^24 integers with T = 1 72 ms in 16 tiles, 89 in 256).
 uint32_t linear_shrink(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
   const sv_config &k = c->cfg;
   uint64_t bits = 0;
-  for (const RangeSpec &s : specs)
+  bool lists = false;
+  for (const RangeSpec &s : specs) {
     if (s.hi > s.lo) bits += (s.hi - s.lo) / 2;
+    lists |= s.list_cap && !s.sieve_only;
+  }
+  const uint64_t enough = lists && k.record_k_threshold <= 3 ? 16 : 3ull * (uint64_t)c->num_sms / 2;
   uint32_t n = 0;
   while (k.tile_log2 - n > 15 && k.margin_log2 - 1 + 3 < k.tile_log2 - n &&
-         specs.size() + (bits >> (k.tile_log2 - n)) < 2ull * (uint64_t)c->num_sms)
+         specs.size() + (bits >> (k.tile_log2 - n)) < enough)
     ++n;
   return n;
 }

@@ -12,9 +12,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("threads", [544, 608, 864, 992])
 def test_halved_blocks_are_whole_warps(orc, threads):
-    # 2^24 odd n in tiles of 2^16 are 257 tiles, fewer than two per SM: halved once
+    # 160 tiles of 2^16 odd n, fewer than three for two SMs: halved once
     lo = (1 << 44) + 12345
-    hi = lo + (1 << 25)
+    hi = lo + 160 * (1 << 17)
     o = orc.verify_range(lo, hi, per_n=True)
     with Verifier(max_hi=1 << 45, tile_log2=16, threads=threads) as v:
         assert_same_range(v.verify_range(lo, hi), o, per_n=False)
@@ -25,6 +25,18 @@ def test_halved_blocks_are_whole_warps(orc, threads):
 
 def test_halved_default_tiles(orc):
     lo = (1 << 47) + 1
-    hi = lo + (1 << 28)
+    hi = lo + 160 * (1 << 20)
     with Verifier(max_hi=1 << 48, threads=544) as v:
         assert_same_range(v.verify_range(lo, hi), orc.verify_range(lo, hi), per_n=False)
+
+
+@pytest.mark.parametrize("T", [2, 3, 4, 6])
+@pytest.mark.parametrize("tiles", [1, 15, 16, 226, 227, 228])
+def test_around_the_halving(orc, T, tiles):
+    # tiles of 2^16 odd n where the halving starts and stops
+    lo = (1 << 44) + 12345
+    hi = lo + tiles * (1 << 17) - 1000
+    with Verifier(max_hi=1 << 45, tile_log2=16, record_k_threshold=T) as v:
+        o = orc.verify_range(lo, hi, per_n=True, list_cap=1 << 22, list_k_threshold=T)
+        assert_same_range(v.verify_range(lo, hi, list_cap=1 << 22), o, per_n=False)
+        assert_same_range(v.verify_range(lo, hi, list_cap=1 << 22, per_n=True), o)
