@@ -228,7 +228,11 @@ Geometry make_geometry(const sv_ctx *c, uint64_t span_bits = 0, size_t n_ranges 
 // ones, down to 64 threads, until there are two tiles per SM or no range
 // would be cut any more: a tile's time is nearly proportional to its
 // size, and SMs without a tile idle, but a smaller block only does the work of
-// an uncut short range with fewer threads.
+// an uncut short range with fewer threads.  A sparse prime costs every tile the
+// same, whatever its size, so there are at most eight per thread (a bucket
+// threshold of 2^14, 1900 primes, and 2^24 integers: 46 us a call, 56 with 16
+// per thread, 78 with blocks of 64 threads regardless; the default's 171 primes
+// never bind).
 uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, const Workspace &ws) {
   const sv_config &k = c->cfg;
   if (k.record_k_threshold <= 5 || ws.force_general || k.stamp_primes != 4 || k.tile_log2 < 15 || k.tile_log2 > 19 ||
@@ -245,7 +249,9 @@ uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, co
   uint32_t S = k.threads;
   if (margin * 8 > 32ull * kStreamRun * S) return 0;  // the margin would be most of the window
   if (stream_smem(S, kMaxSparsePrimes) + stream_static_smem() + 1024 > c->smem_optin) return 0;
-  while (S > 64 && margin * 16 <= 32ull * kStreamRun * S / 2 && longest + margin > 32ull * kStreamRun * S / 2 &&
+  const uint32_t sparse = std::min<uint32_t>(primes_upto(c, k.large_prime_min), kMaxSparsePrimes);  // (at most)
+  while (S > 64 && sparse <= 8 * (S / 2) && margin * 16 <= 32ull * kStreamRun * S / 2 &&
+         longest + margin > 32ull * kStreamRun * S / 2 &&
          specs.size() + bits / (32ull * kStreamRun * S - margin) < 2ull * (uint64_t)c->num_sms)
     S /= 2;
   return S;

@@ -40,3 +40,13 @@ def test_around_the_halving(orc, T, tiles):
         o = orc.verify_range(lo, hi, per_n=True, list_cap=1 << 22, list_k_threshold=T)
         assert_same_range(v.verify_range(lo, hi, list_cap=1 << 22), o, per_n=False)
         assert_same_range(v.verify_range(lo, hi, list_cap=1 << 22, per_n=True), o)
+
+
+@pytest.mark.parametrize("large_prime_min", [3500, 8192, 1 << 14, 1 << 20])
+@pytest.mark.parametrize("log2_len", [18, 20, 24, 26])
+def test_many_sparse_primes(orc, large_prime_min, log2_len):
+    # the stream layout's block stops shrinking at eight sparse primes per thread
+    lo = (1 << 44) + 12345
+    hi = lo + (1 << log2_len) + 999
+    with Verifier(max_hi=1 << 45, large_prime_min=large_prime_min) as v:
+        assert_same_range(v.verify_range(lo, hi), orc.verify_range(lo, hi), per_n=False)
