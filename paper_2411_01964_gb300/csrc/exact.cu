@@ -190,21 +190,33 @@ constexpr uint32_t kMaxDivisors = 16;  // a product of 16 odd primes exceeds 2^6
 
 // A block per point, its threads striding the primes (U per thread and step,
 // their loads in flight together), and K exponents at a time: with few points,
-// so that one pass over the primes mostly suffices.
+// so that one pass over the primes mostly suffices.  A point below `small`
+// needs few primes, and the block's barriers would be most of its time: the
+// warps of the first blocks take those, one each.
 template <int K, int U>
 __global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const uint64_t *pts, uint64_t count,
-                                                            uint8_t *out) {
+                                                            uint64_t small, uint8_t *out) {
   __shared__ uint32_t bad, n_div[K];   // bad: bit j, p^2 divides the j-th value
   __shared__ uint64_t div_inv[K][kMaxDivisors];
   __shared__ uint32_t found;
   __shared__ uint64_t n_s;
   const uint32_t tid = threadIdx.x, T = blockDim.x;
-  for (uint64_t e = blockIdx.x; e < count; e += gridDim.x) {
-    if (tid == 0) n_s = pts[e];  // (perhaps in host memory: read once)
-    __syncthreads();
-    const uint64_t n = n_s;
-    uint32_t k = 0;
-    if (n >= 3 && (n & 1ull)) {
+  const uint64_t e = blockIdx.x;    // a block per point
+  if (tid == 0) n_s = pts[e];       // (perhaps in host memory: read once)
+  {
+    const uint64_t ew = e * (T >> 5) + (tid >> 5);
+    const uint64_t n = ew < count ? pts[ew] : ~0ull;
+    if (n < small) {
+      const uint32_t k = n >= 3 && (n & 1ull) ? warp_min_k_from(n, 1, pt) : 0u;
+      if ((tid & 31u) == 0) out[ew] = (uint8_t)k;
+    }
+  }
+  __syncthreads();
+  const uint64_t n = n_s;
+  if (n < small) return;
+  uint32_t k = 0;
+  {
+    if (n & 1ull) {
       for (uint32_t k0 = 1;; k0 += K) {
         __syncthreads();  // the previous round's results have been read
         if (tid == 0) {
@@ -262,9 +274,8 @@ __global__ void __launch_bounds__(1024) points_block_kernel(PrimeTab pt, const u
       }
       k = found;
     }
-    if (tid == 0) out[e] = (uint8_t)k;
-    __syncthreads();  // found is read above before the next point resets it
   }
+  if (tid == 0) out[e] = (uint8_t)k;
 }
 
 // Many points: a warp takes kSlots points at a time and walks the primes once
@@ -279,43 +290,47 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
   const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t small_p = lane < pt.n_div ? pt.p[lane] : 0ull;
   const uint64_t small_inv = lane < pt.n_div ? pt.inv[lane] : 0ull, small_lim = lane < pt.n_div ? pt.lim[lane] : 0ull;
-  uint64_t s[kSlots], r[kSlots], e[kSlots];  // value, its cofactor so far, point index
-  uint32_t k[kSlots];                        // exponent under test; 0: the slot takes a new point
+  // value n - 2^k, its cofactor so far, point index (~0: none left)
+  uint64_t s[kSlots], r[kSlots], e[kSlots];
+  uint32_t k[kSlots];  // exponent under test; 0: the slot takes a new point
   uint64_t next = gw;
+  auto take = [&](int j) {
+    k[j] = 1;
+    e[j] = next < count ? next : ~0ull;
+    s[j] = next < count ? pts[next] - 2u : 0ull;
+    if (next < count) next += nw;
+  };
 #pragma unroll
-  for (int j = 0; j < kSlots; ++j) k[j] = 0, s[j] = r[j] = 1, e[j] = ~0ull;
+  for (int j = 0; j < kSlots; ++j) k[j] = 0;
   for (;;) {
     bool live = false;
+    // new points for the slots without one, their loads in flight together
+#pragma unroll
+    for (int j = 0; j < kSlots; ++j)
+      if (k[j] == 0) take(j);
 #pragma unroll
     for (int j = 0; j < kSlots; ++j) {
       // the next value of this slot that passes the first 32 primes
       for (;;) {
-        if (k[j] == 0) {
-          e[j] = next;
-          if (next >= count) {  // no point left: the slot idles (s = 1 has no divisor)
-            e[j] = ~0ull;
-            s[j] = r[j] = 1;
-            break;
-          }
-          next += nw;
-          k[j] = 1;
+        if (e[j] == ~0ull) {  // the slot idles (s = 1 has no divisor)
+          s[j] = r[j] = 1;
+          break;
         }
-        const uint64_t n = pts[e[j]];
+        const uint64_t n = s[j] + (1ull << k[j]);
         if (n < 3 || !(n & 1ull)) {
           if (lane == 0) out[e[j]] = 0;
-          k[j] = 0;
+          take(j);
           continue;
         }
         if (k[j] >= 63 || (1ull << k[j]) >= n) {
           if (lane == 0) out[e[j]] = kFailK;
-          k[j] = 0;
+          take(j);
           continue;
         }
-        s[j] = n - (1ull << k[j]);
         const uint64_t t = s[j] * small_inv;
         const bool div = small_p && t <= small_lim;
         if (__any_sync(0xFFFFFFFFu, div && t * small_inv <= small_lim)) {
-          ++k[j];
+          s[j] -= 1ull << k[j]++;
           continue;
         }
         uint32_t m = __ballot_sync(0xFFFFFFFFu, div);
@@ -334,12 +349,23 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
 #pragma unroll
     for (int j = 0; j < kSlots; ++j) top = s[j] > top ? s[j] : top;
     uint32_t bad = 0;
-    // the primes to walk: those with p^3 <= top
+    // the primes to walk: those with p^3 <= top, none if the last of the first
+    // 32 is above; 32 probes a step, first 32 primes apart, then over the rest
+    // of the table (at most five loads one behind the other; halving the table
+    // took seventeen)
     uint32_t n_walk = 0;
-    for (uint32_t hi = pt.n_div; n_walk < hi;) {
-      const uint32_t mid = (n_walk + hi) >> 1;
-      if (cube_le(pt.word[mid].p, top)) n_walk = mid + 1u;
-      else hi = mid;
+    if (__all_sync(0xFFFFFFFFu, small_p && cube_le((uint32_t)small_p, top))) {
+      n_walk = 32;
+      bool near = true;
+      for (uint32_t len = min(pt.n_div - 32u, 1024u); len;) {
+        const uint32_t step = (len + 31u) >> 5, probe = lane * step;
+        const bool in = probe < len && cube_le(pt.word[n_walk + probe].p, top);
+        const uint32_t b = (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, in));  // (primes ascend)
+        if (b == 0) break;
+        n_walk += (b - 1u) * step + 1u;
+        len = near && b == 32u ? pt.n_div - n_walk : min(step - 1u, len - (b - 1u) * step - 1u);
+        near = false;
+      }
     }
     auto walk = [&](auto short_test) {
       constexpr bool kShort = decltype(short_test)::value;
@@ -381,7 +407,7 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
         if (lane == 0) out[e[j]] = (uint8_t)k[j];
         k[j] = 0;
       } else {
-        ++k[j];
+        s[j] -= 1ull << k[j]++;
       }
     }
   }
@@ -392,19 +418,25 @@ __global__ void __launch_bounds__(256) points_warp_kernel(PrimeTab pt, const uin
 // prime and value, a quarter of the logic rate).  One warp per point, with two
 // 64-bit products, 64-bit compares and two votes per 32 primes, took 962 us on
 // the device for 65536 points; the high word of the 64-bit product alone 372;
-// the 32-bit test 213.  1024 points: 21 us before the 32-bit test, 19 now.
-// The lines, with both sides measured: a block of 1024 threads per point while
-// two fit every SM (304 points: 11 us; blocks of 256 with two exponents 15);
-// those (7218 points: 66 us, four points per warp 66; 2048: 26 and 52) up to 48
-// points per SM; then a warp per four points (16384 points: 70 us, blocks 138).
+// the 32-bit test 193.
+// The lines, with both sides measured, n near 2^50: a block of 1024 threads per
+// point while two fit every SM (304 points: 13 us; blocks of 256 with two
+// exponents 15); those (7296 points: 59 us, four points per warp 66; 2048: 23
+// and 52) up to 48 points per SM; then a warp per four points (16384 points: 68
+// us, blocks 138).
+// What counts as a small point depends on how long the blocks queue: up to eight
+// blocks per SM all are resident and a block is as fast as a warp from 2^20 on
+// (1024 points below 2^30: 7 us either way); 2000 points below 2^30 take 8 us by
+// warps and 10 in blocks, 5000 below 2^36 15 and 17, below 2^20 7 and 15.
 cudaError_t launch_points(PrimeTab pt, const uint64_t *pts, uint64_t count, uint8_t *out, uint32_t num_sms,
                           cudaStream_t st) {
   if (count == 0) return cudaSuccess;
   const uint64_t sms = num_sms;
+  const uint64_t small = 1ull << (count <= 8 * sms ? 20 : count <= 20 * sms ? 34 : 38);
   if (count <= 2 * sms)
-    points_block_kernel<4, 2><<<(uint32_t)count, 1024, 0, st>>>(pt, pts, count, out);
+    points_block_kernel<4, 2><<<(uint32_t)count, 1024, 0, st>>>(pt, pts, count, small, out);
   else if (count <= 48 * sms)
-    points_block_kernel<2, 4><<<(uint32_t)count, 256, 0, st>>>(pt, pts, count, out);
+    points_block_kernel<2, 4><<<(uint32_t)count, 256, 0, st>>>(pt, pts, count, small, out);
   else
     points_warp_kernel<<<(uint32_t)std::min<uint64_t>((count + 8 * kSlots - 1) / (8 * kSlots), 4 * sms), 256, 0, st>>>(
         pt, pts, count, out);
