@@ -264,18 +264,19 @@ uint32_t stream_threads(const sv_ctx *c, const std::vector<RangeSpec> &specs, co
 // two SMs on, the halves come to four on some SM, as much as two whole tiles:
 // the per-n output of 2^28 integers, 257 tiles, 78 us whole and 90 halved, of
 // 220 * 2^20, 211 tiles, 78 and 68; lists with T = 5 57 and 77, 56 and 56.)
-// Lists with T <= 3 hold 2% of the n and more and are sorted by the host, which
-// scatters the entries of as many tiles as arrive together: sixteen then (all
-// odd n of 2^24 integers with T = 1 72 ms in 16 tiles, 89 in 256).
+// Lists with T <= 3 hold 2% of the n and more, whose count is bound by one
+// address, and are sorted by the host, which scatters the entries of as many
+// tiles as arrive together: sixteen then (all odd n of 2^24 integers with T = 1
+// 72 ms in 16 tiles, 89 in 256; counted only 5.2 and 5.5 ms).
 uint32_t linear_shrink(const sv_ctx *c, const std::vector<RangeSpec> &specs) {
   const sv_config &k = c->cfg;
   uint64_t bits = 0;
-  bool lists = false;
+  bool scan = false;
   for (const RangeSpec &s : specs) {
     if (s.hi > s.lo) bits += (s.hi - s.lo) / 2;
-    lists |= s.list_cap && !s.sieve_only;
+    scan |= !s.sieve_only;
   }
-  const uint64_t enough = lists && k.record_k_threshold <= 3 ? 16 : 3ull * (uint64_t)c->num_sms / 2;
+  const uint64_t enough = scan && k.record_k_threshold <= 3 ? 16 : 3ull * (uint64_t)c->num_sms / 2;
   uint32_t n = 0;
   while (k.tile_log2 - n > 15 && k.margin_log2 - 1 + 3 < k.tile_log2 - n &&
          specs.size() + (bits >> (k.tile_log2 - n)) < enough)
