@@ -179,7 +179,7 @@ def tile_source_sha() -> str:
 def measured_traffic(n_odd: int):
     """DRAM bytes per launch of the tile kernel from the committed ncu capture,
     scaled by odd n; None when the kernel source changed since the capture."""
-    p = os.path.join(ROOT, "profiles", "tile_kernel_C2_traffic.json")
+    p = os.path.join(ROOT, "profiles", "stream_kernel_C2_traffic.json")
     if not os.path.exists(p):
         return None
     with open(p) as f:

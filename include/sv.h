@@ -74,14 +74,15 @@ typedef struct sv_config {
     uint32_t margin_log2;        /* look-back below each tile, in integers: W = 2^margin_log2
                                     (6..tile_log2+1).  n - 2^k with 2^k <= W is read from the
                                     tile's own window; larger k go to the exact straggler test */
-    uint32_t threads;            /* threads per CTA of the tile kernel (256, 512 or 1024) */
+    uint32_t threads;            /* threads per CTA of the tile kernel: a multiple of 32 from 128 to 1024
+                                    (launches of few tiles take smaller blocks) */
     uint32_t large_prime_min;    /* lower bound of the bucket threshold: primes from the threshold on
                                     are delivered through per-tile buckets.  The library raises the
                                     threshold to about sqrt(range length / 128) and keeps at most 2048
                                     primes between the dense ones and it */
     uint32_t bucket_capacity;    /* entries per tile bucket (grown automatically on overflow) */
     uint32_t record_k_threshold; /* T: every n with mink(n) >= T is listed (default 6) */
-    uint32_t ctas_per_sm;        /* resident tile CTAs per SM (1 or 2) */
+    uint32_t ctas_per_sm;        /* resident tile CTAs per SM (1..4) */
     uint32_t stamp_primes;       /* how many of the smallest odd primes (3, 5, 7, ...) are applied as
                                     computed word patterns instead of atomic strikes: 2, 4, 6 or 8 */
     uint64_t list_capacity;      /* device list entries per range (grown on overflow) */
@@ -179,7 +180,8 @@ sv_status sv_get_config(const sv_ctx *ctx, sv_config *out);
  * Algorithm 1 needs every prime 3 <= p < sqrt(end) (Sec. 3).  Builds, on the
  * device, the table of all odd primes p <= isqrt(max_hi - 1) with the
  * constants the kernels use, and keeps it resident.  max_hi <= 2^62.  Calling
- * it again with a larger max_hi rebuilds the table; a smaller one is a no-op.
+ * it again with a larger max_hi rebuilds the table (also between a launch and
+ * its fetch and while requests are served); a smaller one is a no-op.
  * Errors: SV_EINVAL, SV_ERANGE, SV_ENOMEM, SV_ECUDA.
  */
 sv_status sv_init_primes(sv_ctx *ctx, uint64_t max_hi);

@@ -148,7 +148,7 @@ struct Workspace {
   uint32_t strag_cap = 1u << 16;
   uint32_t bucket_cap = 0;
   bool any_per_n = false;
-  bool ordered = false;        // the planned launch produces ordered lists (tile kernel mode 0)
+  bool ordered = false;        // the planned launch produces ordered lists (their entries staged per tile)
   bool force_general = false;  // repeat with the unordered list path (a tile's staging overflowed)
   bool search_all = false;     // repeat with the first occurrences of k <= 5 searched in every tile
   bool all_from_bitmap = false;  // every range reads its windows from a bitmap: no bucket fill

@@ -8,7 +8,8 @@
 namespace sv {
 
 // ---------------------------------------------------------------------------
-// The ordered list (mode 0).  The launch's tiles are cut into blocks of 128,
+// The ordered list (staged by stream_kernel and by modes 0 and 2 of the linear
+// tile kernel).  The launch's tiles are cut into blocks of 128,
 // one thread per tile (small blocks, so that a launch's tiles spread over
 // the SMs); a tile's place in its range's list is the number of
 // entries its range staged in the tiles before it: the block's inclusive

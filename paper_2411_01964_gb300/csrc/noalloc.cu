@@ -6,8 +6,10 @@
 // this library would fail; latency-critical loops, because cudaMalloc and
 // cudaFree can synchronise the whole device and take milliseconds; and
 // services whose memory budget is fixed when they start.  This entry point
-// runs the same kernels as sv_verify_range, but every piece of scratch memory
-// they need (launch header, range descriptor, result slot, tile buckets,
+// runs the range path in the linear layout (tiles.cu: the general scan, on whole
+// tiles of the configured size; the stream layout and ordered lists stage
+// entries per tile, for which the scratch has no room).  Every piece of scratch
+// memory it needs (launch header, range descriptor, result slot, tile buckets,
 // straggler queue, list and failure arenas) is carved out of one file-scope
 // __device__ array of kScratchBytes.  It calls no cudaMalloc, cudaFree,
 // cudaMallocHost or other allocating routine; results are copied into the

@@ -30,7 +30,7 @@ enum : uint32_t {
   kStTimeout = 1u << 4,         // a bounded wait for a bulk copy ran out (SV_ETIMEDOUT)
 };
 
-// List entries (mink >= T) a tile stages for the ordered list (mode 0): the
+// List entries (mink >= T) a tile stages for the ordered list: the
 // tile kernel's shared buffer and the stride of the per-tile staging slots.
 constexpr uint32_t kStageCap = 128;
 
@@ -207,7 +207,7 @@ struct StragArgs {
   const Straggler *strag;
   uint32_t strag_cap;
   uint32_t rec_t;
-  // ordered lists (mode 0): a straggler's list entry joins its tile's staged entries
+  // ordered lists: a straggler's list entry joins its tile's staged entries
   uint64_t *stage_n;    // null: append to the list directly
   uint8_t *stage_k;
   uint32_t *stage_cnt;
@@ -216,7 +216,7 @@ struct StragArgs {
   uint64_t tw_inv;
 };
 
-// The ordered list (mode 0): each range's staged entries, tile by tile and
+// The ordered list: each range's staged entries, tile by tile and
 // ascending within a tile, into its list region; list_count = the total.
 struct CompactArgs {
   const ReqDesc *reqs;
