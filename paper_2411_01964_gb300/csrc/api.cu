@@ -716,7 +716,10 @@ sv_status enqueue_graph(sv_ctx *c, const Geometry &g, Workspace &ws, cudaStream_
     if (timed)
       for (cudaEvent_t &ev : lg->ev)
         if (!ev && cudaEventCreate(&ev) != cudaSuccess) return SV_ECUDA;
-    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SV_ECUDA;
+    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();  // (not left behind: the next launch's check would report it)
+      return SV_ECUDA;
+    }
     cudaError_t e = cudaMemcpyAsync(ws.io.p, ws.h_io.p, in_bytes, cudaMemcpyHostToDevice, st);
     // sized for the buffers (the kernel reads the launch's sizes from the header)
     if (!e && init)

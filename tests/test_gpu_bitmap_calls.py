@@ -33,3 +33,14 @@ def test_legacy_stream(orc):
     with Verifier(max_hi=1 << 41, stream=1) as v:
         assert_bitmap(v, orc)
         assert_bitmap(v, orc)
+
+
+def test_a_refused_capture_leaves_no_error(orc):
+    # a range on the legacy stream is refused; the next calls are unaffected
+    with Verifier(max_hi=1 << 41, stream=1) as v:
+        with pytest.raises(B.SvError) as e:
+            v.verify_range(LO, HI)
+        assert e.value.status == B.SV_ECUDA
+        assert_bitmap(v, orc)
+    with Verifier(max_hi=1 << 41) as v:
+        assert v.verify_range(LO, HI).hist == orc.verify_range(LO, HI).hist
